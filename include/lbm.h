@@ -111,9 +111,10 @@ typedef struct {
                               (1 when no range is given).                                   */
     int usolve_chebyshev;  /* 1: Chebyshev acceleration of the sweeps for the spectrum [0, g] of
                               the iteration (g as for usolve_omega; needs the density range),
-                              about half the sweeps of the best plain relaxation; it falls
-                              back to plain sweeps within a solve if the residual grows.  The
-                              fixed point, and so the result up to the tolerance, is unchanged */
+                              about half the sweeps of the best plain relaxation on noise.
+                              Solves of smooth flows open with plain sweeps, which are the
+                              faster there, and a solve whose residual grows, or stalls near
+                              the tolerance, ends with them.  The fixed point, and so the result up to the tolerance, is unchanged */
 } lbm_params;
 
 typedef struct {

@@ -723,7 +723,9 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
             smax = std::fmax(smax, std::fabs(4.0 / 3.0 * std::sin(x) - std::sin(2.0 * x) / 6.0));
         }
         dv.s2max = smax * smax;
-        dv.cheb = params->usolve_chebyshev ? 1 : 0;  // the bound of each solve comes from its density range
+        // the bound of each solve comes from its density range.  16-bit storages stay Chebyshev throughout:
+        // their tolerance is far above the rounding of u, and 6 sweeps became 5 at best
+        dv.cheb = params->usolve_chebyshev ? (s->kt.ssize == 2 ? 2 : 1) : 0;
     }
     fill_phys<float>(dv.pf, dv, *eos);
     fill_phys<double>(dv.pd, dv, *eos);

@@ -23,7 +23,7 @@ struct UsolveState {
     int iter;                       // sweeps of the solve in progress
     int iters_last;                 // sweeps of the last finished solve
     int iters_max;                  // largest sweep count since init
-    double resid_last;              // final residual of the last finished solve
+    double resid_last;              // residual of the last sweep: after a solve, its final one
     int converged;                  // 1 once the last solve met its tolerance
     int running;                    // 1 from k_us_begin until the control kernel stops the loop
     long long sweeps_total;         // sweeps since the last reset
@@ -33,15 +33,30 @@ struct UsolveState {
     double cheb_sigma, cheb_delta;  // this solve's spectrum [1 - g, 1] of I - A (theta = 1 - g/2)
     double gain;                    // this solve's bound g, from the density range of the state
     double resid_min;               // smallest residual of the solve so far (divergence guard)
-    int mode;                       // 1: Chebyshev acceleration, 0: plain relaxation
+    int mode;                       // 1: Chebyshev sweeps, 2: plain sweeps of a Chebyshev solve, 0: plain
+                                    // relaxation
     int wsel;                       // pair 0: the warm-start buffer holding the newest j~ (see jwp)
     int tma;                        // 1 once a sweep of this solve loaded planes by tensor copies
+    int opened;                     // 1: this solve (after it: the last one) opened with plain sweeps
 };
 
 // planes ahead of the one in work whose per-site inputs the collision and derivative
 // kernels prefetch into L2 (measured at 256^3)
 constexpr int kCollideLead = 1;
 constexpr int kDerivsLead = 1;
+
+// Plain sweeps inside Chebyshev-accelerated solves (32- and 64-bit storages).  J multiplies smooth
+// modes by almost zero, so on the smooth residual of a steady flow one plain sweep does what takes
+// Chebyshev five; on noise Chebyshev gains a factor 4 per sweep and plain 2.  A solve opens with plain
+// sweeps when the last one, opened by Chebyshev, took kPlainOpen to kPlainOpenMost sweeps, or opened
+// plainly and took fewer than kPlainOpen; it goes on plainly while that halves the residual, and
+// within kPlainNear tolerances.  A Chebyshev solve that no longer halves its residual within
+// kStallNear tolerances ends plainly: u of size 0.03 rounds at 2e-9 in FP32, and updates of 1.6
+// residuals met that rounding at the 5e-9 tolerance.  Longer solves (the noisy start of a quench)
+// stay Chebyshev from first to last: ended plainly, they took 4 % fewer sweeps but left twice the
+// error against FP64.
+constexpr int kPlainOpen = 4, kPlainOpenMost = 5;
+constexpr double kPlainNear = 8.0, kStallNear = 2.0;
 
 // slots of the density-range reduction (spread so that block atomics do not contend)
 constexpr int kRangeSlots = 64;
@@ -106,7 +121,8 @@ struct DevSim {
     double tol, rtol;
     double omega;                    // relaxation of the u-solve sweep (1 = the plain iteration);
                                      // 0: 2/(2 - g) with g the bound of each solve
-    int cheb;                        // Chebyshev acceleration of the sweeps
+    int cheb;                        // Chebyshev acceleration of the sweeps: 1 with plain sweeps where they
+                                     // are the faster (kPlainOpen), 2 throughout, 0 none
     double s2max;                    // max over k of |s(k)|^2 of the first-derivative symbol (1D)
     void* dvec[2];                   // U [3][N]: previous update of the u-solve, pair 0 and 1
     int maxit;

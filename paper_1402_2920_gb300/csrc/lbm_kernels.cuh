@@ -558,6 +558,15 @@ static __device__ double frozen_gain(const DevSim& p, double rho)
     return p.d * p.s2max / 12.0 * fmax(3.0 * cs2 - DP, cs2);
 }
 
+// First step of a Chebyshev semi-iteration from the current iterate: x += r / theta.
+static __device__ __forceinline__ void cheb_first(UsolveState& u)
+{
+    u.mode = 1;
+    u.cheb_rho = 1.0 / u.cheb_sigma;
+    u.c1 = 0.0;
+    u.c2 = 1.0 / (1.0 - u.cheb_delta);
+}
+
 // One warp (lane 0..31) per solve: the reductions are spread over the lanes (one thread took
 // 22 us per step, most of it in the 17 FP64 gain evaluations one after the other).
 static __device__ void b_us_begin(const DevSim& p, int pair, int lane)
@@ -597,11 +606,19 @@ static __device__ void b_us_begin(const DevSim& p, int pair, int lane)
     u.running = 1;
     u.tma = 0;
     u.resid_min = 1e300;
-    if (p.cheb) {  // first Chebyshev step: x += r / theta
-        u.mode = 1;
-        u.cheb_rho = 1.0 / u.cheb_sigma;
+    // Whether this solve opens with plain sweeps (see kPlainOpen in lbm_common.h), from the run's last
+    // solve, which pair 1 reads too: what lbm_fields does depends on the run's state alone.
+    const UsolveState& run = p.us[0];
+    const bool plain = p.cheb == 1 && (run.opened ? run.iters_last < kPlainOpen
+                                                  : run.iters_last >= kPlainOpen && run.iters_last <= kPlainOpenMost);
+    u.opened = plain ? 1 : 0;
+    u.resid_last = 1e300;
+    if (plain) {
+        u.mode = 2;
         u.c1 = 0.0;
-        u.c2 = 1.0 / (1.0 - 0.5 * g);
+        u.c2 = 1.0;
+    } else if (p.cheb) {
+        cheb_first(u);
     } else {       // plain relaxation x += omega r (omega = 0: 2/(2 - g))
         u.mode = 0;
         u.c1 = 0.0;
@@ -627,24 +644,38 @@ static __device__ bool b_us_ctl(const DevSim& p, int pair)
     else if (stop && !conv) atomicOr(p.status, STB_USOLVE_CAP);
     u.resid_bits = 0ull;
     u.jmax_bits = 0ull;
-    // coefficients of the next sweep (Chebyshev semi-iteration for the real spectrum
-    // [1 - g, 1] of I - A); a residual four times above the best one so far means the
-    // spectral bound was too small: continue with plain relaxation
-    if (u.mode == 1 && !bad && r > 4.0 * u.resid_min) u.mode = 0;
-    if (u.mode == 1) {
-        const double rn = 1.0 / (2.0 * u.cheb_sigma - u.cheb_rho);
-        u.c1 = rn * u.cheb_rho;
-        u.c2 = 2.0 * rn / u.cheb_delta;
-        u.cheb_rho = rn;
-    } else if (p.cheb) {  // fell back from Chebyshev: plain sweeps
-        u.c1 = 0.0;
-        u.c2 = 1.0;
+    // Coefficients of the next sweep: Chebyshev semi-iteration for the real spectrum [1 - g, 1] of
+    // I - A, or plain sweeps, whose update is the residual itself.  resid_last holds the residual
+    // of the sweep before.  A residual four times above the best one so far means the spectral bound
+    // was too small: plain sweeps from there on (mode 0).
+    if (p.cheb) {
+        const double lim = p.tol + p.rtol * jm;
+        const bool halved = r <= 0.5 * u.resid_last;
+        if (u.mode == 1 && !bad && r > 4.0 * u.resid_min) u.mode = 0;
+        bool plain = u.mode == 0;
+        if (u.opened)  // plain as long as it pays, and near the tolerance
+            plain = plain || u.iter == 1 || r <= kPlainNear * lim || (u.mode == 2 && halved);
+        else if (p.cheb == 1)  // a Chebyshev update is 1.6 residuals: near the tolerance it can stall on
+                               // the rounding of u where a plain one would end
+            plain = plain || u.mode == 2 || (r <= kStallNear * lim && !halved);
+        if (plain) {
+            u.mode = u.mode == 0 ? 0 : 2;
+            u.c1 = 0.0;
+            u.c2 = 1.0;
+        } else if (u.mode == 2) {
+            cheb_first(u);
+        } else {
+            const double rn = 1.0 / (2.0 * u.cheb_sigma - u.cheb_rho);
+            u.c1 = rn * u.cheb_rho;
+            u.c2 = 2.0 * rn / u.cheb_delta;
+            u.cheb_rho = rn;
+        }
     }
+    u.resid_last = r;
     u.resid_min = r < u.resid_min ? r : u.resid_min;
     if (stop) {
         u.iters_last = u.iter;
         u.iters_max = u.iter > u.iters_max ? u.iter : u.iters_max;
-        u.resid_last = r;
         u.converged = conv ? 1 : 0;
         u.running = 0;
     }
