@@ -474,16 +474,19 @@ dim3 tile_grid(const lbm_sim* s)
                 s->d == 3 ? (s->dev.nz + s->dev.zb - 1) / s->dev.zb : 1);
 }
 
-// z-slab depth of the tiled kernels.  A CTA marches zb planes plus its halo (4 planes; the sweep 9
-// phases), and the grid's tiles_xy * ceil(nz / zb) CTAs run in waves of resident CTAs per SM x SMs.
-// A last wave that fills the GPU only in part leaves SMs idle for a whole march, so on grids of two
-// waves or more the depth in [24, 48] is taken that minimises the sum over the tiled kernels of
-// waves x (zb + halo) x the kernel's time per CTA-plane (measured at 256^3 on GB300: force 1.9,
-// sweep 2.0 x two sweeps per step, derivatives 2.6, collision 6.7 units).  At 256^3 on 152 SMs
-// this gives 37 (1792 CTAs: four waves of the sweep's 456 resident CTAs, where 32 gave 2048 CTAs,
-// 4.5 waves); measured, the step's tiled kernels ran 2 to 5 % faster.  Smaller grids keep 32.
-// LBM_TILE_Z=<n> in the environment at lbm_create sets the depth (any depth gives the same
-// results, bit for bit).
+// z-slab depth of the tiled kernels.  A CTA marches zb planes plus its halo, and the grid's
+// tiles_xy * ceil(nz / zb) CTAs run in waves of (resident CTAs per SM) x SMs.  Deep slabs repeat
+// less halo; shallow ones give a small lattice enough CTAs to fill the chip, and a last wave that
+// is nearly empty costs as much as a full one.  The depth taken minimises the modelled time of a
+// step with three sweeps,
+//   sum over kernels of calls x (zb + halo) x (full waves x l[resident] + l[CTAs per SM of the last wave]),
+// with l[r] the time (us) a CTA takes per plane when r share an SM and halo the cost of a CTA's
+// other planes in the same unit, both fitted to cubes of 16^3 to 192^3 at depths 2 to 48 on GB300
+// (the model is within 10 % of those measurements).  Measured, us per step of force + 3 sweeps +
+// derivatives + collision against the depth of 32 of before: 32^3 359 -> 70, 64^3 377 -> 118, 96^3 406 -> 264,
+// 160^3 1129 -> 1002; 256^3 keeps 37.  With FP64 fields or sweeps the CTAs of an SM share its FP64 units,
+// so l grows with r (48^3 FP64: 4.9 -> 0.78 ms).  LBM_TILE_Z=<n> in the environment at lbm_create
+// sets the depth (any depth gives the same results, bit for bit).
 int choose_zb(const lbm_sim* s)
 {
     if (s->d != 3) return 1;
@@ -497,37 +500,41 @@ int choose_zb(const lbm_sim* s)
     int nsm = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess || nsm < 1) {
         (void)cudaGetLastError();
-        return 32;
+        return nz < 32 ? nz : 32;
     }
+    constexpr int RMAX = 4;
+    const bool f64 = s->kt.tsize == 8 || s->kt.usize == 8;
     struct Kern {
         const void* fn;
         size_t smem;
-        int halo;
-        double w;
-    } ks[4] = {{s->kt.force, s->kt.smem_force, 4, 1.9},
-               {s->sweep, s->kt.smem_sweep, 9, 4.0},
-               {s->kt.derivs, s->kt.smem_derivs, 4, 2.6},
-               {s->kt.collide, s->kt.smem_collide, 4, 6.7}};
-    long long slots[4];
-    for (int k = 0; k < 4; ++k) {
+        double calls, halo, l[RMAX];
+        double l64;  // per plane and resident CTA with FP64 arithmetic
+        int slots;
+    } ks[4] = {{s->kt.force, s->kt.smem_force, 1, 2.0, {0.9, 1.2, 1.5, 1.9}, 6.0, 1},
+               {s->sweep, s->kt.smem_sweep, 3, 6.0, {1.3, 1.65, 2.2, 2.9}, 16.6, 1},
+               {s->kt.derivs, s->kt.smem_derivs, 1, 1.5, {1.8, 2.2, 2.9, 3.9}, 31.0, 1},
+               {s->kt.collide, s->kt.smem_collide, 1, 0.5, {3.3, 6.6, 9.9, 13.2}, 60.0, 1}};
+    for (Kern& k : ks) {
         int r = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, ks[k].fn, s->kt.tile_threads, ks[k].smem) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k.fn, s->kt.tile_threads, k.smem) != cudaSuccess) {
             (void)cudaGetLastError();
             r = 1;
         }
-        slots[k] = (long long)(r > 0 ? r : 1) * nsm;
+        k.slots = r < 1 ? 1 : r > RMAX ? RMAX : r;
+        if (f64)
+            for (int q = 0; q < RMAX; ++q) k.l[q] = k.l64 * (q + 1);
     }
-    auto cost = [&](int zb) {
+    int best = nz < 32 ? nz : 32;
+    double cbest = 1e300;
+    for (int zb = 1; zb <= 48 && zb <= nz; ++zb) {
+        if ((nz + zb - 1) / zb > 65535) continue;  // gridDim.z
         const long long ctas = txy * ((nz + zb - 1) / zb);
         double c = 0.0;
-        for (int k = 0; k < 4; ++k) c += ks[k].w * double((ctas + slots[k] - 1) / slots[k]) * (zb + ks[k].halo);
-        return c;
-    };
-    if (nz <= 32 || txy * ((nz + 31) / 32) < 2 * slots[1]) return nz < 32 ? nz : 32;
-    int best = 32;
-    double cbest = cost(32);
-    for (int zb = 24; zb <= 48 && zb <= nz; ++zb) {
-        const double c = cost(zb);
+        for (const Kern& k : ks) {
+            const long long full = ctas / ((long long)k.slots * nsm), rem = ctas % ((long long)k.slots * nsm);
+            const double waves = double(full) * k.l[k.slots - 1] + (rem ? k.l[(rem + nsm - 1) / nsm - 1] : 0.0);
+            c += k.calls * (zb + k.halo) * waves;
+        }
         if (c < cbest * (1.0 - 1e-9)) {
             best = zb;
             cbest = c;
