@@ -71,8 +71,8 @@ namespace {
 
 int nblocks(long long N, int block) { return int((N + block - 1) / block); }
 
-// grid of the tiled kernels: one CTA per TX x TY column tile and z-slab
-dim3 tile_grid(const lbm_sim* s);
+// grid of a tiled kernel: one CTA per TX x TY column tile and z-slab
+dim3 tile_grid(const lbm_sim* s, TiledKernel k);
 dim3 moments_grid(const lbm_sim* s);
 int moments_block(const lbm_sim* s);
 cudaError_t launch_moments(const lbm_sim* s, DevSim dv, int src, int pair);
@@ -187,6 +187,7 @@ void fill_phys(Phys<T>& q, const DevSim& dv, const lbm_eos& e)
     q.cf_h2 = T(0.5 / (c0 * c0));
     q.cf_h3 = T(1.0 / (6.0 * c0 * c0 * c0));
     q.cj = T((1.0 - g) * c0);
+    for (int k = 0; k < 8; ++k) q.w0h2[k] = T(dv.w0[k] * 0.5 / (c0 * c0));
 }
 
 // warm-start j~ buffers: two for the start extrapolated from the last two steps
@@ -214,6 +215,17 @@ size_t bytes_per_site(int lattice, int storage, size_t* ssize_out = nullptr)
     // populations (two buffers), rest planes, rho - rho0, j0', f, aux; u iterates (2 x 2),
     // warm-start j~ (two buffers with the extrapolated start) and the two Chebyshev update vectors
     return 2 * Q * ssize + rest + wref + tsize * (1 + 3 + 3 + naux) + usize * (4 * 3 + 2 * 3 + 2 * 3);
+}
+
+// whether x-neighbouring sites (2k, 2k + 1) are aligned words of every field plane
+bool pairs_of_sites(const int64_t dims[3]) { return dims[0] % 2 == 0; }
+// Whether the pairwise collision takes tiles of 64 x 4 sites (else 32 x 8): where they pad nx by at most a
+// fifth more.  Measured, 64 / 32 wide: 256^3 1.17 / 1.59 ms, 192^3 0.50 / 0.56, 160^3 (padded by a fifth)
+// 0.333 / 0.329, 128^3 0.155 / 0.160, 96^3 (a third) 0.087 / 0.076, 48^3 14 / 15 us.
+bool wide_tiles(const int64_t dims[3])
+{
+    const int64_t w32 = (dims[0] + 31) / 32 * 32, w64 = (dims[0] + 63) / 64 * 64;
+    return 5 * w64 <= 6 * w32;
 }
 
 int validate(int lattice, const int64_t dims[3], int storage)
@@ -261,11 +273,10 @@ int add_step(lbm_sim* s, cudaGraph_t g, cudaGraphNode_t dep, int src, cudaGraphN
         void* a[] = {&dv, &src, &pair};
         LBM_CK(add_kernel(g, &n1, s->kt.moments, moments_grid(s), moments_block(s), a, d0, nd0));
     }
-    const dim3 TG = tile_grid(s);
-    const int TB = s->kt.tile_threads;
+    const TileShape* ts = s->kt.tile;
     {
         void* a[] = {&dv, &pair};
-        LBM_CK(add_kernel(g, &n2, s->kt.force, TG, TB, a, &n1, 1, s->kt.smem_force));
+        LBM_CK(add_kernel(g, &n2, s->kt.force, tile_grid(s, TK_FORCE), ts[TK_FORCE].threads, a, &n1, 1, s->kt.smem_force));
     }
     {
         void* a[] = {&dv, &pair};
@@ -283,17 +294,17 @@ int add_step(lbm_sim* s, cudaGraph_t g, cudaGraphNode_t dep, int src, cudaGraphN
     {
         cudaGraphNode_t b1, b3;
         void* a1[] = {&dv, &pair};
-        LBM_CK(add_kernel(body, &b1, s->sweep, TG, TB, a1, nullptr, 0, s->kt.smem_sweep));
+        LBM_CK(add_kernel(body, &b1, s->sweep, tile_grid(s, TK_SWEEP), ts[TK_SWEEP].threads, a1, nullptr, 0, s->kt.smem_sweep));
         void* a3[] = {&dv, &pair, &h, &one};
         LBM_CK(add_kernel(body, &b3, s->kt.us_ctl, dim3(1), 1, a3, &b1, 1));
     }
     {
         void* a[] = {&dv};
-        LBM_CK(add_kernel(g, &n5, s->kt.derivs, TG, TB, a, &nc, 1, s->kt.smem_derivs));
+        LBM_CK(add_kernel(g, &n5, s->kt.derivs, tile_grid(s, TK_DERIVS), ts[TK_DERIVS].threads, a, &nc, 1, s->kt.smem_derivs));
     }
     {
         void* a[] = {&dv, &src};
-        LBM_CK(add_kernel(g, &n6, s->kt.collide, TG, TB, a, &n5, 1, s->kt.smem_collide));
+        LBM_CK(add_kernel(g, &n6, s->kt.collide, tile_grid(s, TK_COLLIDE), ts[TK_COLLIDE].threads, a, &n5, 1, s->kt.smem_collide));
     }
     *last = n6;
     return LBM_OK;
@@ -341,10 +352,12 @@ cudaError_t launch(const lbm_sim* s, const void* fn, int grid, int block, A... a
 }
 
 template <class... A>
-cudaError_t launch_tiled(const lbm_sim* s, const void* fn, size_t smem, A... args)
+cudaError_t launch_tiled(const lbm_sim* s, TiledKernel k, A... args)
 {
+    const void* fn[kTiled] = {s->kt.force, s->sweep, s->kt.derivs, s->kt.collide};
+    const size_t smem[kTiled] = {s->kt.smem_force, s->kt.smem_sweep, s->kt.smem_derivs, s->kt.smem_collide};
     void* a[] = {&args...};
-    return cudaLaunchKernel(fn, tile_grid(s), dim3(s->kt.tile_threads), a, smem, s->stream);
+    return cudaLaunchKernel(fn[k], tile_grid(s, k), dim3(s->kt.tile[k].threads), a, smem[k], s->stream);
 }
 
 int read_status(lbm_sim* s, int* bits)
@@ -467,80 +480,85 @@ cudaError_t launch_moments(const lbm_sim* s, DevSim dv, int src, int pair)
     return cudaLaunchKernel(s->kt.moments, moments_grid(s), dim3(moments_block(s)), a, 0, s->stream);
 }
 
-dim3 tile_grid(const lbm_sim* s)
+dim3 tile_grid(const lbm_sim* s, TiledKernel k)
 {
-    const int* t = s->kt.tile;
-    return dim3((s->dev.nx + t[0] - 1) / t[0], (s->dev.ny + t[1] - 1) / t[1],
-                s->d == 3 ? (s->dev.nz + s->dev.zb - 1) / s->dev.zb : 1);
+    const TileShape& t = s->kt.tile[k];
+    const int zb = s->dev.zb[k];
+    return dim3((s->dev.nx + t.tx - 1) / t.tx, (s->dev.ny + t.ty - 1) / t.ty, s->d == 3 ? (s->dev.nz + zb - 1) / zb : 1);
 }
 
-// z-slab depth of the tiled kernels.  A CTA marches zb planes plus its halo, and the grid's
+// z-slab depth of each tiled kernel.  A CTA marches zb planes plus its halo, and the grid's
 // tiles_xy * ceil(nz / zb) CTAs run in waves of (resident CTAs per SM) x SMs.  Deep slabs repeat
 // less halo; shallow ones give a small lattice enough CTAs to fill the chip, and a last wave that
-// is nearly empty costs as much as a full one.  The depth taken minimises the modelled time of a
-// step with three sweeps,
-//   sum over kernels of calls x (zb + halo) x (full waves x l[resident] + l[CTAs per SM of the last wave]),
+// is nearly empty costs as much as a full one.  The depth taken minimises the modelled time
+//   (zb + halo) x (full waves x l[resident] + l[CTAs per SM of the last wave]),
 // with l[r] the time (us) a CTA takes per plane when r share an SM and halo the cost of a CTA's
 // other planes in the same unit, both fitted to cubes of 16^3 to 192^3 at depths 2 to 48 on GB300
 // (the model is within 10 % of those measurements).  Measured, us per step of force + 3 sweeps +
-// derivatives + collision against the depth of 32 of before: 32^3 359 -> 70, 64^3 377 -> 118, 96^3 406 -> 264,
-// 160^3 1129 -> 1002; 256^3 keeps 37.  With FP64 fields or sweeps the CTAs of an SM share its FP64 units,
+// derivatives + collision against the one depth of 32 of before: 32^3 359 -> 70, 64^3 377 -> 118, 96^3 406 -> 264,
+// 160^3 1129 -> 1002.  With FP64 fields or sweeps the CTAs of an SM share its FP64 units,
 // so l grows with r (48^3 FP64: 4.9 -> 0.78 ms).  LBM_TILE_Z=<n> in the environment at lbm_create
-// sets the depth (any depth gives the same results, bit for bit).
-int choose_zb(const lbm_sim* s)
+// sets the depth of all (any depth gives the same results, bit for bit).
+void choose_zb(lbm_sim* s)
 {
-    if (s->d != 3) return 1;
-    const int nz = s->dev.nz;
+    DevSim& dv = s->dev;
+    for (int& zb : dv.zb) zb = 1;
+    if (s->d != 3) return;
+    const int nz = dv.nz;
+    for (int& zb : dv.zb) zb = nz < 32 ? nz : 32;
     if (const char* env = std::getenv("LBM_TILE_Z")) {
         const int v = std::atoi(env);
-        if (v >= 1) return v < nz ? v : nz;
+        if (v >= 1) {
+            for (int& zb : dv.zb) zb = v < nz ? v : nz;
+            return;
+        }
     }
-    const int* t = s->kt.tile;
-    const long long txy = (long long)((s->dev.nx + t[0] - 1) / t[0]) * ((s->dev.ny + t[1] - 1) / t[1]);
     int nsm = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess || nsm < 1) {
         (void)cudaGetLastError();
-        return nz < 32 ? nz : 32;
+        return;
     }
     constexpr int RMAX = 4;
     const bool f64 = s->kt.tsize == 8 || s->kt.usize == 8;
     struct Kern {
         const void* fn;
         size_t smem;
-        double calls, halo, l[RMAX];
+        double halo, l[RMAX];
         double l64;  // per plane and resident CTA with FP64 arithmetic
-        int slots;
-    } ks[4] = {{s->kt.force, s->kt.smem_force, 1, 2.0, {0.9, 1.2, 1.5, 1.9}, 6.0, 1},
-               {s->sweep, s->kt.smem_sweep, 3, 6.0, {1.3, 1.65, 2.2, 2.9}, 16.6, 1},
-               {s->kt.derivs, s->kt.smem_derivs, 1, 1.5, {1.8, 2.2, 2.9, 3.9}, 31.0, 1},
-               {s->kt.collide, s->kt.smem_collide, 1, 0.5, {3.3, 6.6, 9.9, 13.2}, 60.0, 1}};
-    for (Kern& k : ks) {
+    } ks[kTiled] = {{s->kt.force, s->kt.smem_force, 2.0, {0.9, 1.2, 1.5, 1.9}, 6.0},
+                    {s->sweep, s->kt.smem_sweep, 6.0, {1.3, 1.65, 2.2, 2.9}, 16.6},
+                    {s->kt.derivs, s->kt.smem_derivs, 1.5, {1.8, 2.2, 2.9, 3.9}, 31.0},
+                    {s->kt.collide, s->kt.smem_collide, 0.5, {3.3, 6.6, 9.9, 13.2}, 60.0}};
+    if (s->kt.derivs == s->kt.pair_derivs) {  // the kernels on pairs of sites
+        const double ld[RMAX] = {1.5, 2.0, 2.55, 3.4}, lc[RMAX] = {2.75, 5.0, 7.5, 10.0};
+        for (int m = 0; m < RMAX; ++m) ks[TK_DERIVS].l[m] = ld[m], ks[TK_COLLIDE].l[m] = lc[m];
+        ks[TK_DERIVS].halo = 1.3;
+        ks[TK_COLLIDE].halo = 0.3;
+    }
+    for (int q = 0; q < kTiled; ++q) {
+        Kern& k = ks[q];
+        const TileShape& t = s->kt.tile[q];
+        const long long txy = (long long)((dv.nx + t.tx - 1) / t.tx) * ((dv.ny + t.ty - 1) / t.ty);
         int r = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k.fn, s->kt.tile_threads, k.smem) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k.fn, t.threads, k.smem) != cudaSuccess) {
             (void)cudaGetLastError();
             r = 1;
         }
-        k.slots = r < 1 ? 1 : r > RMAX ? RMAX : r;
+        r = r < 1 ? 1 : r > RMAX ? RMAX : r;
         if (f64)
-            for (int q = 0; q < RMAX; ++q) k.l[q] = k.l64 * (q + 1);
-    }
-    int best = nz < 32 ? nz : 32;
-    double cbest = 1e300;
-    for (int zb = 1; zb <= 48 && zb <= nz; ++zb) {
-        if ((nz + zb - 1) / zb > 65535) continue;  // gridDim.z
-        const long long ctas = txy * ((nz + zb - 1) / zb);
-        double c = 0.0;
-        for (const Kern& k : ks) {
-            const long long full = ctas / ((long long)k.slots * nsm), rem = ctas % ((long long)k.slots * nsm);
-            const double waves = double(full) * k.l[k.slots - 1] + (rem ? k.l[(rem + nsm - 1) / nsm - 1] : 0.0);
-            c += k.calls * (zb + k.halo) * waves;
-        }
-        if (c < cbest * (1.0 - 1e-9)) {
-            best = zb;
-            cbest = c;
+            for (int m = 0; m < RMAX; ++m) k.l[m] = k.l64 * (m + 1);
+        double cbest = 1e300;
+        for (int zb = 1; zb <= 48 && zb <= nz; ++zb) {
+            if ((nz + zb - 1) / zb > 65535) continue;  // gridDim.z
+            const long long ctas = txy * ((nz + zb - 1) / zb), slots = (long long)r * nsm;
+            const long long full = ctas / slots, rem = ctas % slots;
+            const double c = (zb + k.halo) * (double(full) * k.l[r - 1] + (rem ? k.l[(rem + nsm - 1) / nsm - 1] : 0.0));
+            if (c < cbest * (1.0 - 1e-9)) {
+                dv.zb[q] = zb;
+                cbest = c;
+            }
         }
     }
-    return best;
 }
 
 // S1-S8 on the current populations with the scratch j~ pair; host-driven loop.
@@ -550,12 +568,12 @@ int run_fields(lbm_sim* s)
     const int B = s->kt.block, G = nblocks(dv.N, B);
     const int pair = 1;
     LBM_CK(launch_moments(s, dv, s->cur, pair));
-    LBM_CK(launch_tiled(s, s->kt.force, s->kt.smem_force, dv, pair));
+    LBM_CK(launch_tiled(s, TK_FORCE, dv, pair));
     LBM_CK(launch(s, s->kt.us_begin, 1, 32, dv, pair));
     cudaGraphConditionalHandle h{};
     const int no = 0;
     for (int it = 0; it < s->dev.maxit + 1; ++it) {
-        LBM_CK(launch_tiled(s, s->sweep, s->kt.smem_sweep, dv, pair));
+        LBM_CK(launch_tiled(s, TK_SWEEP, dv, pair));
         LBM_CK(launch(s, s->kt.us_ctl, 1, 1, dv, pair, h, no));
         UsolveState u;
         LBM_CK(cudaMemcpyAsync(&u, &dv.us[1], sizeof(u), cudaMemcpyDeviceToHost, s->stream));
@@ -682,6 +700,19 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
     bool ok = lattice == LBM_D3Q59 ? get_kernels_d3q59(params->storage, us64, read_pops, &s->kt)
                                    : get_kernels_d2q21(params->storage, us64, read_pops, &s->kt);
     if (!ok) { delete s; return LBM_E_INVALID_ARG; }
+    // the kernels on pairs of sites need pairs that stay aligned words: nx even
+    if (s->kt.pair_derivs && pairs_of_sites(dims)) {
+        KernelTable& kt = s->kt;
+        kt.derivs = kt.pair_derivs;
+        kt.kb_derivs = kt.kb_pair_derivs;
+        kt.tile[TK_DERIVS] = kt.tile_pair_derivs;
+        kt.smem_derivs = kt.smem_pair_derivs;
+        const PairCollide& c = kt.pair_collide[wide_tiles(dims) ? 1 : 0];
+        kt.collide = c.collide;
+        kt.kb_collide = c.kb_collide;
+        kt.tile[TK_COLLIDE] = c.tile;
+        kt.smem_collide = c.smem;
+    }
 
     DevSim& dv = s->dev;
     dv.lattice = lattice;
@@ -736,6 +767,18 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
     }
     fill_phys<float>(dv.pf, dv, *eos);
     fill_phys<double>(dv.pd, dv, *eos);
+    for (int k = 0; k < nshell; ++k) {
+        // velocities of shell k as multiples of {-1, 0, 1}^3 ones
+        int m = 1;
+        for (int i = 1; i < s->Q; ++i) {
+            const int ks = lattice == LBM_D3Q59 ? Lat<1>::shell(i) : Lat<0>::shell(i);
+            const int cx = lattice == LBM_D3Q59 ? Lat<1>::cx(i) : Lat<0>::cx(i);
+            if (ks == k && std::abs(cx) > m) m = std::abs(cx);
+        }
+        dv.pc.wh2[k] = float(dv.w0[k] * m * m * 0.5 / (cs0 * cs0));
+        dv.pc.wl[k] = float(dv.w0[k] * m);
+        dv.pc.wh3[k] = float(dv.w0[k] * m * m * m / (6.0 * cs0 * cs0 * cs0));
+    }
 
     const size_t N = size_t(dv.N);
     const size_t T = s->kt.tsize, U = s->kt.usize, SS = s->kt.ssize;
@@ -800,7 +843,7 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
         dv.aligned16 = ok ? 1 : 0;
     }
     setup_sweep_maps(s);
-    dv.zb = choose_zb(s);
+    choose_zb(s);
     // well-defined contents before the first lbm_init
     for (int b = 0; b < 2; ++b) {
         const size_t wbytes = dv.wref[b] ? size_t(lattice == LBM_D3Q59 ? 8 : 6) * N * sizeof(float) : 0;
@@ -875,10 +918,10 @@ int step_direct(lbm_sim* s)
     const int pair = 0, no = 0, src = s->cur;
     cudaGraphConditionalHandle h{};
     LBM_CK(launch_moments(s, dv, src, pair));
-    LBM_CK(launch_tiled(s, s->kt.force, s->kt.smem_force, dv, pair));
+    LBM_CK(launch_tiled(s, TK_FORCE, dv, pair));
     LBM_CK(launch(s, s->kt.us_begin, 1, 32, dv, pair));
     for (int it = 0; it < dv.maxit + 1; ++it) {
-        LBM_CK(launch_tiled(s, s->sweep, s->kt.smem_sweep, dv, pair));
+        LBM_CK(launch_tiled(s, TK_SWEEP, dv, pair));
         LBM_CK(launch(s, s->kt.us_ctl, 1, 1, dv, pair, h, no));
         UsolveState u;
         LBM_CK(cudaMemcpyAsync(&u, &dv.us[0], sizeof(u), cudaMemcpyDeviceToHost, s->stream));
@@ -888,8 +931,8 @@ int step_direct(lbm_sim* s)
                          (long long)s->steps, u.iter, u.running ? u.resid_min : u.resid_last, u.mode, u.c1, u.c2);
         if (!u.running) break;
     }
-    LBM_CK(launch_tiled(s, s->kt.derivs, s->kt.smem_derivs, dv));
-    LBM_CK(launch_tiled(s, s->kt.collide, s->kt.smem_collide, dv, src));
+    LBM_CK(launch_tiled(s, TK_DERIVS, dv));
+    LBM_CK(launch_tiled(s, TK_COLLIDE, dv, src));
     s->cur ^= 1;
     return LBM_OK;
 }
@@ -1066,7 +1109,7 @@ int lbm_profile(lbm_sim* s, int reps, double* ms_out, int n)
     LBM_CK(cudaEventCreate(&e1));
     // the scratch u-solve pair; the collision writes the spare population buffer
     LBM_CK(launch_moments(s, dv, src, pair));
-    LBM_CK(launch_tiled(s, s->kt.force, s->kt.smem_force, dv, pair));
+    LBM_CK(launch_tiled(s, TK_FORCE, dv, pair));
     LBM_CK(launch(s, s->kt.us_begin, 1, 32, dv, pair));
     int rc = LBM_OK;
     for (int k = 0; k < 5 && rc == LBM_OK; ++k) {
@@ -1075,10 +1118,10 @@ int lbm_profile(lbm_sim* s, int reps, double* ms_out, int n)
             cudaError_t e = cudaSuccess;
             switch (k) {
             case 0: e = launch_moments(s, dv, src, pair); break;
-            case 1: e = launch_tiled(s, s->kt.force, s->kt.smem_force, dv, pair); break;
-            case 2: e = launch_tiled(s, s->sweep, s->kt.smem_sweep, dv, pair); break;
-            case 3: e = launch_tiled(s, s->kt.derivs, s->kt.smem_derivs, dv); break;
-            case 4: e = launch_tiled(s, s->kt.collide, s->kt.smem_collide, dv, src); break;
+            case 1: e = launch_tiled(s, TK_FORCE, dv, pair); break;
+            case 2: e = launch_tiled(s, TK_SWEEP, dv, pair); break;
+            case 3: e = launch_tiled(s, TK_DERIVS, dv); break;
+            case 4: e = launch_tiled(s, TK_COLLIDE, dv, src); break;
             }
             if (e != cudaSuccess) rc = LBM_E_CUDA;
         }
@@ -1228,7 +1271,8 @@ struct Batch {
 int batch_key(int lattice, const int64_t dims[3], const lbm_params& prm)
 {
     const bool us64 = prm.storage == LBM_STORE_F64 || prm.usolve_precision == LBM_USOLVE_F64;
-    const int combo = ((lattice * 16 + prm.storage) * 2 + (us64 ? 1 : 0)) * 2 + (prm.gamma != 0.0 ? 1 : 0);
+    const int combo = (((lattice * 16 + prm.storage) * 2 + (us64 ? 1 : 0)) * 2 + (prm.gamma != 0.0 ? 1 : 0)) * 3 +
+                      (pairs_of_sites(dims) ? (wide_tiles(dims) ? 2 : 1) : 0);
     int64_t n = dims[0] * dims[1] * (lattice == LBM_D3Q59 ? dims[2] : 1);
     int size_class = 0;
     while (n >= 4) {
@@ -1262,7 +1306,8 @@ int build_batch_graph(Batch* b)
     DevSim* sims = b->d_sims;
     BatchWork* w = b->d_work;
     int pair = 0;
-    const int TB = kt.tile_threads;
+    const int FB = kt.tile[TK_FORCE].threads, SB = kt.tile[TK_SWEEP].threads, DB = kt.tile[TK_DERIVS].threads,
+              CB = kt.tile[TK_COLLIDE].threads;
     const int MB = kt.local_ref ? kMomentsRowBlock : kt.block;
     cudaGraphNode_t n0, n1, n2, n3, nc, n5, n6, n7;
     {
@@ -1275,7 +1320,7 @@ int build_batch_graph(Batch* b)
     }
     {
         void* a[] = {&sims, &w, &pair};
-        LBM_CK(add_kernel(b->g, &n2, kt.kb_force, dim3(resident_grid(kt.kb_force, TB, kt.smem_force)), TB, a, &n1, 1,
+        LBM_CK(add_kernel(b->g, &n2, kt.kb_force, dim3(resident_grid(kt.kb_force, FB, kt.smem_force)), FB, a, &n1, 1,
                           kt.smem_force));
     }
     {
@@ -1294,19 +1339,19 @@ int build_batch_graph(Batch* b)
         cudaGraph_t body = cp.conditional.phGraph_out[0];
         cudaGraphNode_t b1, b2;
         void* a1[] = {&sims, &w, &pair};
-        LBM_CK(add_kernel(body, &b1, kt.kb_sweep, dim3(resident_grid(kt.kb_sweep, TB, kt.smem_sweep)), TB, a1, nullptr, 0,
+        LBM_CK(add_kernel(body, &b1, kt.kb_sweep, dim3(resident_grid(kt.kb_sweep, SB, kt.smem_sweep)), SB, a1, nullptr, 0,
                           kt.smem_sweep));
         void* a2[] = {&sims, &w, &pair, &h};
         LBM_CK(add_kernel(body, &b2, kt.kb_us_ctl, dim3(1), 32, a2, &b1, 1));
     }
     {
         void* a[] = {&sims, &w};
-        LBM_CK(add_kernel(b->g, &n5, kt.kb_derivs, dim3(resident_grid(kt.kb_derivs, TB, kt.smem_derivs)), TB, a, &nc, 1,
+        LBM_CK(add_kernel(b->g, &n5, kt.kb_derivs, dim3(resident_grid(kt.kb_derivs, DB, kt.smem_derivs)), DB, a, &nc, 1,
                           kt.smem_derivs));
     }
     {
         void* a[] = {&sims, &w};
-        LBM_CK(add_kernel(b->g, &n6, kt.kb_collide, dim3(resident_grid(kt.kb_collide, TB, kt.smem_collide)), TB, a, &n5,
+        LBM_CK(add_kernel(b->g, &n6, kt.kb_collide, dim3(resident_grid(kt.kb_collide, CB, kt.smem_collide)), CB, a, &n5,
                           1, kt.smem_collide));
     }
     {
@@ -1375,7 +1420,7 @@ int batch_launch(Batch* b, const int64_t* steps)
     for (int k = 0; k < kBatchSlots; ++k)
         if (b->slot[k]) nslot = k + 1;
     w.nslot = nslot;
-    w.tstart[0] = 0;
+    for (int q = 0; q < kTiled; ++q) w.tstart[q][0] = 0;
     w.mstart[0] = 0;
     for (int k = 0; k < kBatchSlots; ++k) {
         lbm_sim* s = b->slot[k];
@@ -1385,20 +1430,17 @@ int batch_launch(Batch* b, const int64_t* steps)
         w.live[k] = 0;
         w.todo[k] = int(n);
         w.src[k] = s ? s->cur : 0;
-        int tiles = 0, mblocks = 0;
-        w.tgx[k] = w.tgy[k] = w.mgx[k] = w.mgy[k] = 1;
-        if (s) {
-            b->h_sims[k] = s->dev;
-            const dim3 tg = tile_grid(s), mg = moments_grid(s);
-            w.tgx[k] = int(tg.x);
-            w.tgy[k] = int(tg.y);
-            w.mgx[k] = int(mg.x);
-            w.mgy[k] = int(mg.y);
-            tiles = int(tg.x * tg.y * tg.z);
-            mblocks = int(mg.x * mg.y * mg.z);
+        if (s) b->h_sims[k] = s->dev;
+        for (int q = 0; q < kTiled; ++q) {
+            const dim3 g = s ? tile_grid(s, TiledKernel(q)) : dim3(1, 1, 0);
+            w.tgx[q][k] = int(g.x);
+            w.tgy[q][k] = int(g.y);
+            w.tstart[q][k + 1] = w.tstart[q][k] + int(g.x * g.y * g.z);
         }
-        w.tstart[k + 1] = w.tstart[k] + (k < nslot ? tiles : 0);
-        w.mstart[k + 1] = w.mstart[k] + (k < nslot ? mblocks : 0);
+        const dim3 m = s ? moments_grid(s) : dim3(1, 1, 0);
+        w.mgx[k] = int(m.x);
+        w.mgy[k] = int(m.y);
+        w.mstart[k + 1] = w.mstart[k] + int(m.x * m.y * m.z);
     }
     if (most == 0) return LBM_OK;
     LBM_CK(cudaMemcpyAsync(b->d_sims, b->h_sims, sizeof(DevSim) * size_t(nslot), cudaMemcpyHostToDevice, b->stream));

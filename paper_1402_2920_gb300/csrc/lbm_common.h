@@ -58,6 +58,12 @@ constexpr int kDerivsLead = 1;
 constexpr int kPlainOpen = 4, kPlainOpenMost = 5;
 constexpr double kPlainNear = 8.0, kStallNear = 2.0;
 
+// The tiled kernels: each has its tile, its z-slab depth and so its grid.
+enum TiledKernel { TK_FORCE = 0, TK_SWEEP, TK_DERIVS, TK_COLLIDE, kTiled };
+struct TileShape {
+    int tx, ty, threads;
+};
+
 // slots of the density-range reduction (spread so that block atomics do not contend)
 constexpr int kRangeSlots = 64;
 
@@ -82,7 +88,14 @@ struct Phys {
     T isc[8];                             // 1 / w_k(c_s^2(rho0)): scale of the half storage
     T offc[8];                            // w_k rho0 (FP64) minus off[k] in this precision
     T k1, k2, k3;                         // prefactors of Sigma (two) and Xi' (Sec. VIII, S11)
+    T w0h2[8];                            // w_k(c_s^2(rho0)) cf_h2
     T cf_int, cf_jt, cf_h2, cf_h3, cj;    // (1+g)/(2 cs0), (g-1)/cs0, 1/(2 cs0^2), 1/(6 cs0^3), (1-g) cs0
+};
+
+// Constants of the pairwise collision per shell, m the multiple that the shell's velocities are of their
+// base pairs': w_k(c_s^2(rho0)) times m^2 cf_h2, m and m^3 cf_h3.
+struct PairConst {
+    float wh2[8], wl[8], wh3[8];
 };
 
 // Everything a kernel needs, passed by value (lives in the kernel parameter space).
@@ -131,6 +144,7 @@ struct DevSim {
     double wtheta;                   // warm = 2: j~ start = j~_n + wtheta (j~_n - j~_n-1)
     Phys<float> pf;                  // the same parameters for FP32 arithmetic
     Phys<double> pd;                 // and for FP64 arithmetic
+    PairConst pc;
     // Tensor maps of the sweep's plane loads (TMA) in device memory, valid when tma = 1.
     const struct SweepMaps* tmaps;
     // plane i of population buffer b, pop[b] + i N elements: the collision's stores address their
@@ -146,12 +160,11 @@ struct DevSim {
     void* fpp[3];
     void* jwp[2][3];
     int tma;
-    int zb;  // z planes per CTA of the tiled kernels (3D; 1 in 2D), chosen at creation
+    int zb[kTiled];  // z planes per CTA of each tiled kernel (3D; 1 in 2D), chosen at creation
 };
 
 // The sweep's tensor maps: the u iterates uit[pair][buffer] as {nx, ny, nz, 3} and rho - rho0
-// as {nx, ny, nz}, each loaded in boxes of 40 x 16 sites (the tile with its in-plane halo of 4)
-// of one plane.
+// as {nx, ny, nz}, each loaded in boxes of one plane: the sweep's tile with its in-plane halo of 4.
 struct SweepMaps {
     CUtensorMap u[2][2];
     CUtensorMap rho;
@@ -166,10 +179,17 @@ struct BatchWork {
     int live[kBatchSlots];           // 1: the slot takes the current step
     int src[kBatchSlots];            // its current population buffer
     int todo[kBatchSlots];           // steps it still takes in the running chunk
-    int tstart[kBatchSlots + 1];     // prefix sums of the tiled kernels' tile counts
+    int tstart[kTiled][kBatchSlots + 1];  // prefix sums of each tiled kernel's tile counts
     int mstart[kBatchSlots + 1];     // prefix sums of the moments kernel's block counts
-    int tgx[kBatchSlots], tgy[kBatchSlots];  // tile grid extents in x and y
+    int tgx[kTiled][kBatchSlots], tgy[kTiled][kBatchSlots];  // its grid extents in x and y
     int mgx[kBatchSlots], mgy[kBatchSlots];  // moments grid extents in x and y
+};
+
+// The collision on pairs of x-neighbouring sites: one tile width.
+struct PairCollide {
+    const void *collide, *kb_collide;
+    TileShape tile;
+    size_t smem;
 };
 
 // Kernels of one (lattice, arithmetic, storage, u-solve arithmetic) combination.
@@ -201,8 +221,12 @@ struct KernelTable {
     const void* kb_collide;     // (sims, work)
     const void* kb_step_end;    // (sims, work)
     int block;                // threads per block of the per-site kernels
-    int tile[2];              // TX, TY of the tiled kernels (the z-slab depth is DevSim::zb)
-    int tile_threads;
+    TileShape tile[kTiled];   // of force, sweep, derivs, collide (the z-slab depths are DevSim::zb)
+    // derivs and collide on pairs of x-neighbouring sites, for nx even (null: there are none)
+    PairCollide pair_collide[2];  // tiles 32 and 64 wide
+    const void *pair_derivs, *kb_pair_derivs;
+    TileShape tile_pair_derivs;
+    size_t smem_pair_derivs;
     size_t smem_force, smem_sweep, smem_derivs, smem_collide;  // dynamic shared memory bytes
     size_t tsize, usize, ssize;  // bytes of T, U and the storage type
     size_t rsize;                // bytes of a rest-plane element (0: no separate plane)

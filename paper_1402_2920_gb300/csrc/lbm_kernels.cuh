@@ -805,6 +805,28 @@ __host__ __device__ constexpr bool pair_base(int i)
     return true;
 }
 
+// Multiple m (1, 2, 4) that shell k's velocities are of their base pairs'.
+template <int LAT>
+__host__ __device__ constexpr int shell_multiple(int k)
+{
+    using L = Lat<LAT>;
+    const int i = first_pair_of_shell<LAT>(k);
+    int m = 1;
+    for (int c : {L::cx(i), L::cy(i), L::cz(i)}) m = c < 0 ? (-c > m ? -c : m) : (c > m ? c : m);
+    return m;
+}
+
+// Shell of the velocities m c with c in {-1, 0, 1}^3 and n non-zero components; 0 if there is none.
+template <int LAT>
+__host__ __device__ constexpr int class_shell(int n, int m)
+{
+    using L = Lat<LAT>;
+    for (int i = 1; i < L::Q; i += 2)
+        if ((L::cx(i) != 0) + (L::cy(i) != 0) + (L::cz(i) != 0) == n && shell_multiple<LAT>(L::shell(i)) == m)
+            return L::shell(i);
+    return 0;
+}
+
 // f(integral_constant<int, 0>), ..., f(integral_constant<int, N - 1>) at compile time
 template <int... I, class F>
 __device__ __forceinline__ void static_foreach_impl(std::integer_sequence<int, I...>, F&& f)
@@ -1225,8 +1247,8 @@ __device__ __forceinline__ void b_sweep(const DevSim& p, int pair, const Blk bid
     auto slot = [](int z) { return D == 3 ? (z + 8 * R) % R : 0; };  // z >= -8
     const int tid = threadIdx.x;
     const int x0 = bid.x * TX, y0 = bid.y * TY;
-    const int z0 = D == 3 ? bid.z * p.zb : 0;
-    const int z1 = D == 3 ? min(z0 + p.zb, p.nz) : 1;
+    const int z0 = D == 3 ? bid.z * p.zb[TK_SWEEP] : 0;
+    const int z1 = D == 3 ? min(z0 + p.zb[TK_SWEEP], p.nz) : 1;
     const long long NP = (long long)p.nx * p.ny;  // sites per plane
     const T* drho = cp<T>(p.rho);
     const int cur = p.us[pair].cur;
@@ -1521,6 +1543,108 @@ __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, sizeof(U) == 4 ? 3
     b_sweep<LAT, T, U, TMA>(p, pair, launch_blk());
 }
 
+// ---------------------------------------------------------------------------
+// Packed pairs of floats (Blackwell's FP32x2 instructions): one instruction, one issue slot, two
+// independent IEEE results, each rounded as the scalar instruction rounds it.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long bits2(float2 v) { return reinterpret_cast<const unsigned long long&>(v); }
+__device__ __forceinline__ float2 pair2(unsigned long long v) { return reinterpret_cast<const float2&>(v); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
+    return pair2(r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
+    return pair2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
+    return pair2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)), "l"(bits2(c)));
+    return pair2(r);
+}
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+// The Sec. IV.B first derivative of two points, d1v's operations in d1v's order.
+__device__ __forceinline__ float2 d1v2(float2 m2, float2 m1, float2 p1, float2 p2)
+{
+    return fma2(both(float(2.0 / 3.0)), sub2(p1, m1), mul2(both(-float(1.0 / 12.0)), sub2(p2, m2)));
+}
+// ... along x, of the points in the middle word xc of three consecutive pairs
+__device__ __forceinline__ float2 d1x2(float2 xm, float2 xc, float2 xp)
+{
+    return fma2(both(float(2.0 / 3.0)), make_float2(xc.y - xm.y, xp.x - xc.x),
+                mul2(both(-float(1.0 / 12.0)), sub2(xp, xm)));
+}
+// Equation of state of two sites (see eos_full, cs2_delta).  Every operation is written out, and the psi-sine
+// form is one function that is not inlined, so that a site's result does not depend on which of the
+// two words it has: left to the compiler, the two scalar copies contracted differently in rare cases.
+static __device__ __noinline__ float4 psi_eos(float rho, float rho1, float rho3, float cs2_1, float A, float pi_D,
+                                              float A_pi_D, float AD_pi)
+{
+    float psi = 0.f, dpsi = 0.f, integ = 0.f;
+    if (rho > rho1 && rho < rho3) {
+        const float ph = pi_D * (rho - rho1);
+        const float sn = sinf(ph), cn = cosf(ph);
+        psi = A * sn;
+        dpsi = A_pi_D * cn;
+        integ = AD_pi * (1.f - cn);
+    }
+    const float cs2 = cs2_1 * expf(integ);
+    const float P = rho * cs2, DP = cs2 * (1.f + rho * psi);
+    return make_float4(P, DP, P - rho * DP, rho * (cs2 * psi * (1.f + rho * psi) + cs2 * (psi + rho * dpsi)));
+}
+static __device__ __noinline__ float psi_cs2(float drho, float rho0, float rho1, float pi_D, float ph0_raw, float AD_pi,
+                                             float cs0)
+{
+    constexpr float PI = 3.14159265358979323846f;
+    const float ph_raw = pi_D * (rho0 + drho - rho1);
+    const float ph = fminf(fmaxf(ph_raw, 0.f), 2.f * PI), ph0 = fminf(fmaxf(ph0_raw, 0.f), 2.f * PI);
+    const bool inside = ph == ph_raw && ph0 == ph0_raw;
+    const float dph = inside ? pi_D * drho : ph - ph0;
+    return cs0 * expm1f(AD_pi * 2.f * sinf(0.5f * (ph + ph0)) * sinf(0.5f * dph));
+}
+__device__ __forceinline__ void eos2(const DevSim& p, float2 rho, float2& P, float2& DP, float2& PM, float2& RPP)
+{
+    const Phys<float>& q = p.pf;
+    if (p.eos_kind == 0) {
+        const float2 den = fma2(both(-q.b), rho, both(1.f));
+        const float2 ig = make_float2(1.f / den.x, 1.f / den.y);
+        P = fma2(mul2(rho, both(q.Teos)), ig, mul2(mul2(both(-q.a), rho), rho));
+        DP = fma2(mul2(both(q.Teos), ig), ig, mul2(both(-2.f * q.a), rho));
+        RPP = mul2(rho, fma2(mul2(mul2(both(2.f * q.bT), ig), ig), ig, both(-2.f * q.a)));
+        PM = fma2(mul2(both(-1.f), rho), DP, P);
+    } else {
+        const float4 a = psi_eos(rho.x, q.rho1, q.rho3, q.cs2_1, q.A, q.pi_D, q.A_pi_D, q.AD_pi);
+        const float4 b = psi_eos(rho.y, q.rho1, q.rho3, q.cs2_1, q.A, q.pi_D, q.A_pi_D, q.AD_pi);
+        P = make_float2(a.x, b.x);
+        DP = make_float2(a.y, b.y);
+        PM = make_float2(a.z, b.z);
+        RPP = make_float2(a.w, b.w);
+    }
+}
+// c_s^2(rho) - c_s^2(rho0)
+__device__ __forceinline__ float2 cs2_delta2(const DevSim& p, float2 drho)
+{
+    const Phys<float>& q = p.pf;
+    if (p.eos_kind == 0) {
+        const float2 g = fma2(both(-q.b), drho, both(q.g0)), n = mul2(both(q.b2T_g02), drho);
+        const float2 corr = make_float2(n.x / g.x, n.y / g.y);
+        return fma2(drho, both(q.F0), fma2(drho, both(q.F0lo), mul2(drho, corr)));
+    }
+    return make_float2(psi_cs2(drho.x, q.rho0, q.rho1, q.pi_D, q.ph0, q.AD_pi, q.cs0),
+                       psi_cs2(drho.y, q.rho0, q.rho1, q.pi_D, q.ph0, q.AD_pi, q.cs0));
+}
+
 // S2 (tiled): f = kappa rho d_a lap rho with the third-derivative stencil of Sec. IV.E,
 // j0' = j0 + (h/2) f, and the start of the u-solve u = (j0' + j~)/rho with j~ of the previous
 // step (warm start, Sec. IX item 3) or j~ = 0 (S1).  The CTA marches along z; rho - rho0 of
@@ -1549,8 +1673,8 @@ __device__ __forceinline__ void b_force(const DevSim& p, int pair, const Blk bid
     T* sr = reinterpret_cast<T*>(smem_raw);  // [R][RY][RX]: rho - rho0
     const int tid = threadIdx.x;
     const int x0 = bid.x * TX, y0 = bid.y * TY;
-    const int z0 = D == 3 ? bid.z * p.zb : 0;
-    const int z1 = D == 3 ? min(z0 + p.zb, p.nz) : 1;
+    const int z0 = D == 3 ? bid.z * p.zb[TK_FORCE] : 0;
+    const int z1 = D == 3 ? min(z0 + p.zb[TK_FORCE], p.nz) : 1;
     const long long NP = (long long)p.nx * p.ny;
     const T* drho = cp<T>(p.rho);
     U* u0 = mp<U>(p.uit[pair][p.us[pair].cur]);
@@ -1690,8 +1814,8 @@ __device__ __forceinline__ void b_derivs(const DevSim& p, const Blk bid)
     T* sr = reinterpret_cast<T*>(smem_raw);  // [R][NP][RY][RX]
     const int tid = threadIdx.x, nth = blockDim.x;
     const int x0 = bid.x * TX, y0 = bid.y * TY;
-    const int z0 = D == 3 ? bid.z * p.zb : 0;
-    const int z1 = D == 3 ? min(z0 + p.zb, p.nz) : 1;
+    const int z0 = D == 3 ? bid.z * p.zb[TK_DERIVS] : 0;
+    const int z1 = D == 3 ? min(z0 + p.zb[TK_DERIVS], p.nz) : 1;
     const T* drho = cp<T>(p.rho);
     const U* uu = cp<U>(p.uit[0][p.us[0].cur]);  // S8: the converged u
     constexpr int MR = (RX * RY + TL::THREADS - 1) / TL::THREADS;
@@ -1806,8 +1930,8 @@ __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, sizeof(T) == 4 && 
     T* sr = reinterpret_cast<T*>(smem_raw);  // [R][NP][RY][RX]
     const int tid = threadIdx.x, nth = blockDim.x;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const int z0 = D == 3 ? int(blockIdx.z) * p.zb : 0;
-    const int z1 = D == 3 ? min(z0 + p.zb, p.nz) : 1;
+    const int z0 = D == 3 ? int(blockIdx.z) * p.zb[TK_DERIVS] : 0;
+    const int z1 = D == 3 ? min(z0 + p.zb[TK_DERIVS], p.nz) : 1;
     const T* drho = cp<T>(p.rho);
     const U* uu = cp<U>(p.uit[0][p.us[0].cur]);  // S8: the converged u
     constexpr int MR = (RX * RY + TL::THREADS - 1) / TL::THREADS;
@@ -1939,8 +2063,8 @@ __device__ __forceinline__ void b_collide(const DevSim& p, int src, const Blk bi
     T* sr = reinterpret_cast<T*>(smem_raw);  // [R][NP][RY][RX]
     const int tid = threadIdx.x, nth = blockDim.x;
     const int x0 = bid.x * TX, y0 = bid.y * TY;
-    const int z0 = D == 3 ? bid.z * p.zb : 0;
-    const int z1 = D == 3 ? min(z0 + p.zb, p.nz) : 1;
+    const int z0 = D == 3 ? bid.z * p.zb[TK_COLLIDE] : 0;
+    const int z1 = D == 3 ? min(z0 + p.zb[TK_COLLIDE], p.nz) : 1;
     const T* drho = cp<T>(p.rho);
     const U* uu = cp<U>(p.uit[0][p.us[0].cur]);
     const int ws = p.us[0].wsel;  // the warm-start buffer this step's j~ goes to
@@ -2100,6 +2224,525 @@ __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, 2) k_collide(DevSi
 }
 
 // ---------------------------------------------------------------------------
+// The 3D derivative and collision kernels on pairs of sites (FP32 deviations, nx even)
+// ---------------------------------------------------------------------------
+// (hi, lo) += v of two sites: acc2 in packed instructions
+__device__ __forceinline__ void acc2_2(float2& hi, float2& lo, float2 v)
+{
+    const float2 s = add2(hi, v);
+    const float2 bb = sub2(s, hi);
+    const float2 e = add2(sub2(hi, sub2(s, bb)), sub2(v, bb));
+    hi = s;
+    lo = add2(lo, e);
+}
+
+// Shared memory of the pairwise collision: a ring of the three planes C (halo 2), five planes of the
+// stencil and one in flight, and two stages of the tile's own inputs.
+template <int W>
+struct PairCollidePlan {
+    static constexpr int TX = W, TY = 256 / W, NT = TX * TY / 2, SITES = TX * TY;
+    static constexpr int RX = TX + 4, RY = TY + 4, RP = RX * RY, NP = 3;
+    static constexpr int R = 6;
+    static constexpr int NOWN = 27;  // Sigma's local part (6), Xi' (10), u, j0', f, rho - rho0, rho_lo
+    static constexpr size_t OFF_OWN = size_t(R) * NP * RP * sizeof(float);
+    static constexpr size_t BYTES = OFF_OWN + size_t(2) * NOWN * SITES * sizeof(float);
+};
+
+// Collision and push streaming of the sites (x, y, z) and (x + 1, y, z), x even: collide_tail's
+// formulas, each operation on both sites.  The multiple m of a pair's velocity (base c, 2c or 4c) is a
+// power of two and folds into its shell's constants (PairConst), so that every pair costs
+//   E = aA (c.u)^2 + wh2 Sigma:cc + even0,   O = aI c.u + (wl c.V + wh3 Xi':ccc),   n*_{+-} = E +- O
+// in the base pair's contractions.
+template <int S, bool READ>
+__device__ __forceinline__ void collide_tail_pair(const DevSim& p, int src, int x, int y, int z, int s, float2 drs,
+                                                  float2 lo, float2 rs, const float2 (&u)[3], const float2 (&f)[3],
+                                                  const float2 (&jtl)[3], const float2 (&Sig)[6], const float2 (&Xi)[10])
+{
+    using L = Lat<1>;
+    using C = Codec<S>;
+    static_assert(C::EXACT && !C::SCALED && !C::LOC && C::DEV && sizeof(typename C::type) == 4, "FP32 deviations");
+    static_assert(pairs_opposite<1>(), "velocity table must list opposite pairs");
+    const Phys<float>& q = p.pf;
+    const float2 cs0 = both(q.cs0);
+    const float2 dcs2 = cs2_delta2(p, drs), cs2 = add2(cs0, dcs2);
+    const float2 ics2 = make_float2(1.f / cs2.x, 1.f / cs2.y);
+    const float2 uu = fma2(u[2], u[2], fma2(u[1], u[1], mul2(u[0], u[0])));
+    const float2 A1 = mul2(both(0.5f), mul2(ics2, ics2)), B1 = mul2(both(-0.5f), mul2(uu, ics2));
+    const float2 h2c = mul2(both(-q.cs0), add2(add2(Sig[0], Sig[1]), Sig[2]));  // the c-independent part of h2
+    // c.V gathers the odd terms linear in c: cf_int f + cf_jt j~ - 3 cs0 cf_h3 tr Xi'
+    float2 V[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const float2 t = add2(add2(Xi[sym3<3>(0, 0, b)], Xi[sym3<3>(1, 1, b)]), Xi[sym3<3>(2, 2, b)]);
+        V[b] = fma2(both(-3.f * q.cs0 * q.cf_h3), t, fma2(both(q.cf_jt), jtl[b], mul2(both(q.cf_int), f[b])));
+    }
+    // c_s^2 sums of the weights' difference form (see collide_tail)
+    const float2 s1 = add2(cs2, cs0), s2 = fma2(cs2, s1, mul2(cs0, cs0));
+    // wrapped destination offsets (site indices < 2^31) for the shifts -4, -2, -1, 0, 1, 2, 4.  A pair
+    // stays a pair under even shifts in x (nx is even); under +-1 its sites go to words of two pairs.
+    int ox[7], oy[7], oz[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        const int sh = k == 0 ? -4 : k == 6 ? 4 : k - 3;
+        ox[k] = wrapc(x + sh, p.nx);
+        oy[k] = wrapc(y + sh, p.ny) * p.nx;
+        oz[k] = wrapc(z + sh, p.nz) * p.nx * p.ny;
+    }
+    auto sidx = [](int c) { return c == -4 ? 0 : c == 4 ? 6 : c + 3; };
+    auto put = [&](auto ic, float2 v) {  // population i of both sites to r + c_i
+        constexpr int i = decltype(ic)::value;
+        constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+        float* base = mp<float>(p.popp[src ^ 1][i]);
+        const int row = oy[sidx(cy)] + oz[sidx(cz)];
+        if constexpr (cx % 2 == 0) {
+            __stcs(reinterpret_cast<float2*>(base + (row + ox[sidx(cx)])), v);
+        } else {
+            __stcs(base + (row + ox[sidx(cx)]), v.x);
+            __stcs(base + (row + ox[sidx(cx + 1)]), v.y);
+        }
+    };
+    float2 sh = both(0.f), sl = both(0.f);  // float-pair sums of the stored values
+    // One shell's constants of both sites: what its pairs multiply their contractions by
+    struct ShellC {
+        float2 aA, aI, even0;
+    };
+    auto shell = [&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        const float2 w0k = both(q.w0[k]);
+        const float2 dwk = mul2(dcs2, fma2(both(float(L::wc(k, 3))), s2, fma2(both(float(L::wc(k, 2))), s1, both(float(L::wc(k, 1))))));
+        const float2 wl = add2(w0k, dwk);
+        float2 wr = mul2(wl, rs);
+        // n^eq - w(rho0) rho0 = w rho X + w drho + rho0 (w(s) - w(s0))
+        float2 e = fma2(wr, B1, fma2(wl, drs, mul2(both(q.rho0), dwk)));
+        if (READ) {
+            const float2 omg = both(1.f - q.gamma);
+            e = mul2(omg, e);
+            wr = mul2(omg, wr);
+        }
+        ShellC c;
+        constexpr float m = float(shell_multiple<1>(k));
+        c.even0 = fma2(both(q.w0h2[k]), h2c, e);
+        c.aA = mul2(mul2(wr, both(m * m)), A1);
+        c.aI = mul2(mul2(wr, both(m)), ics2);
+        return c;
+    };
+    auto emit = [&](auto ic, const ShellC& c, float2 uc, float2 uc2, float2 lin, float2 h2, float2 h3) {
+        constexpr int i = decltype(ic)::value;  // the pair (i, i + 1), velocity +m c of the base
+        constexpr int k = L::shell(i);
+        const float2 E = fma2(c.aA, uc2, fma2(both(p.pc.wh2[k]), h2, c.even0));
+        const float2 O = fma2(c.aI, uc, fma2(both(p.pc.wl[k]), lin, mul2(both(p.pc.wh3[k]), h3)));
+        float2 np = add2(E, O), nm = sub2(E, O);
+        if (READ) {
+            const float2 g = both(q.gamma);
+            np = fma2(g, *reinterpret_cast<const float2*>(cp<float>(p.popp[src][i]) + s), np);
+            nm = fma2(g, *reinterpret_cast<const float2*>(cp<float>(p.popp[src][i + 1]) + s), nm);
+        }
+        put(std::integral_constant<int, i>{}, np);
+        put(std::integral_constant<int, i + 1>{}, nm);
+        acc2_2(sh, sl, np);
+        acc2_2(sh, sl, nm);
+    };
+    // The base pairs, direction class by direction class (axes, face diagonals, body diagonals), each
+    // with its multiples, whose shells' constants are made once per class.
+    static_foreach<3>([&](auto cc) {
+        constexpr int n = decltype(cc)::value + 1;  // non-zero components of the class's velocities
+        const ShellC k1 = shell(std::integral_constant<int, class_shell<1>(n, 1)>{});
+        const ShellC k2 = shell(std::integral_constant<int, class_shell<1>(n, 2)>{});
+        ShellC k4 = k2;
+        if constexpr (class_shell<1>(n, 4) != 0) k4 = shell(std::integral_constant<int, class_shell<1>(n, 4)>{});
+        static_foreach<(L::Q - 1) / 2>([&](auto pc) {
+            constexpr int i = 2 * decltype(pc)::value + 1;
+            constexpr int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+            constexpr int nz = (c[0] != 0) + (c[1] != 0) + (c[2] != 0);
+            if constexpr (pair_base<1>(i) && nz == n) {
+                // contractions with c.u, c.V, Sigma:cc, Xi':ccc, the first term of each without its addend
+                float2 uc, lin, h2, h3;
+                bool first = true;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    if (c[a] == 0) continue;
+                    if (first) {
+                        uc = c[a] > 0 ? u[a] : mul2(both(-1.f), u[a]);
+                        lin = c[a] > 0 ? V[a] : mul2(both(-1.f), V[a]);
+                    } else {
+                        uc = c[a] > 0 ? add2(uc, u[a]) : sub2(uc, u[a]);
+                        lin = c[a] > 0 ? add2(lin, V[a]) : sub2(lin, V[a]);
+                    }
+                    first = false;
+                }
+                first = true;
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int b = a; b < 3; ++b) {
+                        const int m = (a == b ? 1 : 2) * c[a] * c[b];
+                        if (m == 0) continue;
+                        const float2 t = Sig[sym2<3>(a, b)];
+                        if (first) h2 = m == 1 ? t : mul2(both(float(m)), t);
+                        else h2 = m == 1 ? add2(h2, t) : fma2(both(float(m)), t, h2);
+                        first = false;
+                    }
+                first = true;
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int b = a; b < 3; ++b)
+#pragma unroll
+                        for (int e = b; e < 3; ++e) {
+                            const int m = ((a == b && b == e) ? 1 : (a == b || b == e) ? 3 : 6) * c[a] * c[b] * c[e];
+                            if (m == 0) continue;
+                            const float2 t = Xi[sym3<3>(a, b, e)];
+                            if (first) h3 = m == 1 ? t : mul2(both(float(m)), t);
+                            else h3 = m == 1 ? add2(h3, t) : m == -1 ? sub2(h3, t) : fma2(both(float(m)), t, h3);
+                            first = false;
+                        }
+                const float2 uc2 = mul2(uc, uc);
+                emit(std::integral_constant<int, i>{}, k1, uc, uc2, lin, h2, h3);
+                constexpr int j2 = pair_multiple<1>(i, 2), j4 = pair_multiple<1>(i, 4);
+                static_assert(j2 >= 0 && j4 >= 0, "multiples of a pair's velocity are listed with its sign");
+                if constexpr (j2 > 0) emit(std::integral_constant<int, j2>{}, k2, uc, uc2, lin, h2, h3);
+                if constexpr (j4 > 0) emit(std::integral_constant<int, j4>{}, k4, uc, uc2, lin, h2, h3);
+            }
+        });
+    });
+    // rest population: the exact pre-collision sum less the stored ones (see collide_tail)
+    auto rest = [&](float th, float tl, float shs, float sls) {
+        float e, rh, h2, l2;
+        two_sum(th, -shs, rh, e);
+        const float rl = __fadd_rn(e, __fsub_rn(tl, sls));
+        two_sum(rh, rl, h2, l2);
+        return make_float2(h2, l2);
+    };
+    const float2 ra = rest(drs.x, lo.x, sh.x, sl.x), rb = rest(drs.y, lo.y, sh.y, sl.y);
+    *reinterpret_cast<float4*>(mp<float2>(p.pop0[src ^ 1]) + s) = make_float4(ra.x, ra.y, rb.x, rb.y);
+}
+
+// S11 (rest) and S12 of the 3D lattice with FP32 deviations and nx even: b_collide on pairs of
+// x-neighbouring sites.  Tiles are 64 x 4 sites, or 32 x 8 where 64 would pad nx by a fifth more.
+//   - Sigma's d_a A + d_g B_ag is d_b q_ab, the divergence that the converged u-solve has already taken:
+//     j~ = -(1/12) d_b q_ab (S5), up to the solve's tolerance.  So A and B (7 of the 26 aux planes) are neither
+//     stored nor read, 12 of the 21 stencils go, and the ring holds C alone (31 KB instead of 104).
+//   - Every instruction serves two sites: packed FP32x2 arithmetic, 64-bit accesses, and 40 of the 58 moving
+//     populations stored as 64-bit words (b_collide: 2,292 thread instructions per site).
+//   - The pair's own 27 inputs come by cp.async into two stages of shared memory, a plane ahead.  Loaded
+//     into registers at their use, they left eight warps waiting: long-scoreboard stalls 2.8 per issue,
+//     and the packed kernel no faster than b_collide.
+//   - Rows of 64 sites give the 59 write streams 256-byte segments, which DRAM takes better than 128-byte ones.
+// Measured: 1.65 (b_collide) -> 1.63 (packed) -> 1.59 (C alone, staged inputs) -> 1.17 ms (64-wide) at 256^3, 223 -> 155 us
+// at 128^3; 372 bytes per site, 0.80 of the measured copy bandwidth at 256^3.  128 x 2 tiles 1.37 ms (halo).
+template <int S, bool READ, int W>
+__device__ __forceinline__ void b_collide_pair(const DevSim& p, int src, const Blk bid)
+{
+    using AL = AuxLayout<3>;
+    using CP = PairCollidePlan<W>;
+    constexpr int TX = CP::TX, TY = CP::TY, NT = CP::NT, RX = CP::RX, RP = CP::RP, NP = CP::NP, R = CP::R;
+    constexpr int HZ = 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* sr = reinterpret_cast<float*>(smem_raw);                // [R][NP][RY][RX]: C
+    float* so = reinterpret_cast<float*>(smem_raw + CP::OFF_OWN);  // [2][NOWN][TY][TX]: own inputs
+    const int tid = threadIdx.x;
+    const int x0 = bid.x * TX, y0 = bid.y * TY;
+    const int z0 = bid.z * p.zb[TK_COLLIDE], z1 = min(z0 + p.zb[TK_COLLIDE], p.nz);
+    const int NPL = p.nx * p.ny;
+    const float* drho = cp<float>(p.rho);
+    const float* uu = cp<float>(p.uit[0][p.us[0].cur]);
+    const int ws = p.us[0].wsel;  // the warm-start buffer this step's j~ goes to
+    // pairs of box columns (the box starts at x0 - 2, an even column): one 8-byte copy each
+    constexpr int NG = RP / 2, MG = (NG + NT - 1) / NT;
+    int goff[MG];
+#pragma unroll
+    for (int m = 0; m < MG; ++m) {
+        const int t = tid + m * NT, gx = t % (RX / 2) * 2, gy = t / (RX / 2);
+        goff[m] = t < NG ? wrapm(x0 - 2 + gx, p.nx) + p.nx * wrapm(y0 - 2 + gy, p.ny) : 0;
+    }
+    auto fetch = [&](int zl, int sl) {
+        const int base = wrapc(zl, p.nz) * NPL;
+        float* dst = sr + sl * NP * RP;
+#pragma unroll
+        for (int m = 0; m < MG; ++m) {
+            const int t = tid + m * NT;
+            if (t < NG) {
+#pragma unroll
+                for (int c = 0; c < NP; ++c) cp_async<8>(dst + c * RP + t * 2, auxp<float>(p, AL::C + c) + (base + goff[m]));
+            }
+        }
+    };
+    const int ix = tid % (TX / 2) * 2, iy = tid / (TX / 2);
+    const int gx = x0 + ix, gy = y0 + iy;
+    const bool in = gx < p.nx && gy < p.ny;
+    const int sxy = gx + p.nx * gy;
+    float* const own = so + iy * TX + ix;
+    auto fetch_own = [&](int z) {  // the pair's own inputs of plane z into stage z & 1
+        if (!in || z < z0 || z >= z1) return;
+        float* dst = own + (z & 1) * CP::NOWN * CP::SITES;
+        const int n = sxy + NPL * z;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) cp_async<8>(dst + c * CP::SITES, auxp<float>(p, AL::SIGL + c) + n);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            cp_async<8>(dst + (16 + a) * CP::SITES, uu + a * p.N + n);
+            cp_async<8>(dst + (19 + a) * CP::SITES, plane<float>(p.j0pp, a) + n);
+            cp_async<8>(dst + (22 + a) * CP::SITES, plane<float>(p.fpp, a) + n);
+        }
+        cp_async<8>(dst + 25 * CP::SITES, drho + n);
+        cp_async<8>(dst + 26 * CP::SITES, cp<float>(p.rho_lo) + n);
+    };
+    int sl = (z0 - HZ + 8 * R) % R;  // ring slot of plane zl (z0 - HZ >= -2)
+    fetch(z0 - HZ, sl);
+    cp_async_commit();
+    for (int zl = z0 - HZ; zl < z1 + HZ; ++zl) {
+        const int zc = zl - HZ;
+        cp_async_wait<0>();  // plane zl and the own inputs of plane zc have landed (this thread's copies)
+        __syncthreads();     // ... and everyone's; the previous pass's reads are done
+        const int sn = sl + 1 == R ? 0 : sl + 1;  // held plane zl - 5, which only the previous pass read
+        if (zl + 1 < z1 + HZ) fetch(zl + 1, sn);
+        fetch_own(zc + 1);
+        cp_async_commit();
+        if (zc >= z0 && in) {
+            const int s = sxy + NPL * zc;
+            const float* ow = own + (zc & 1) * CP::NOWN * CP::SITES;
+            auto ld = [&](int c) { return ld2<float>(ow + c * CP::SITES); };
+            const float2 drs = ld(25);
+            const float2 rs = add2(both(p.pf.rho0), drs);
+            float2 ua[3], f[3], jtl[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                ua[a] = ld(16 + a);
+                f[a] = ld(22 + a);
+                jtl[a] = fma2(rs, ua[a], mul2(both(-1.f), ld(19 + a)));  // j~ = rho u - j0' (S8)
+                *reinterpret_cast<float2*>(plane<float>(p.jwp[ws], a) + s) = jtl[a];  // the next step's warm start
+            }
+            float2 P, DP, PM, RPP;
+            eos2(p, rs, P, DP, PM, RPP);
+            const float* pl[5];  // the pair's word in the planes zc - 2 .. zc + 2
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                const int b = 4 - k, t = sl >= b ? sl - b : sl - b + R;
+                pl[k] = sr + t * NP * RP + (iy + 2) * RX + ix + 2;
+            }
+            float2 dC[3][3];  // d_a C_b
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const float* g = pl[2] + b * RP;
+                dC[0][b] = d1x2(ld2<float>(g - 2), ld2<float>(g), ld2<float>(g + 2));
+                dC[1][b] = d1v2(ld2<float>(g - 2 * RX), ld2<float>(g - RX), ld2<float>(g + RX), ld2<float>(g + 2 * RX));
+                dC[2][b] = d1v2(ld2<float>(pl[0] + b * RP), ld2<float>(pl[1] + b * RP), ld2<float>(pl[3] + b * RP),
+                                ld2<float>(pl[4] + b * RP));
+            }
+            const float k1 = -12.f * p.pf.k1, k2 = p.pf.k2;
+            const float2 trdC = add2(add2(dC[0][0], dC[1][1]), dC[2][2]);
+            const float2 kP = mul2(both(-k2), P), kT = mul2(mul2(both(-k2), PM), trdC);
+            float2 Sig[6];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = a; b < 3; ++b) {
+                    float2 v = fma2(kP, add2(dC[a][b], dC[b][a]), ld(sym2<3>(a, b)));
+                    if (a == b) v = add2(v, kT);
+                    // k1 [u_a (d_b A + d_g B_bg) + u_b (d_a A + d_g B_ag)] with d_a A + d_g B_ag = -12 j~_a
+                    Sig[sym2<3>(a, b)] = fma2(both(k1), fma2(ua[a], jtl[b], mul2(ua[b], jtl[a])), v);
+                }
+            float2 Xi[10];
+#pragma unroll
+            for (int q = 0; q < 10; ++q) Xi[q] = ld(6 + q);
+            collide_tail_pair<S, READ>(p, src, gx, gy, zc, s, drs, ld(26), rs, ua, f, jtl, Sig, Xi);
+        }
+        sl = sn;
+    }
+}
+template <int S, bool READ, int W>
+__global__ void __launch_bounds__(PairCollidePlan<W>::NT, 2) k_collide_pair(DevSim p, int src)
+{
+    b_collide_pair<S, READ, W>(p, src, launch_blk());
+}
+
+// Shared memory of the pairwise derivative kernel: a ring of u, rho - rho0 and c_s^2 - c_s^2(rho0), five planes
+// of the stencil and one in flight.
+struct PairDerivsPlan {
+    static constexpr int TX = 32, TY = 8, NT = TX * TY / 2;
+    static constexpr int RX = TX + 4, RY = TY + 4, RP = RX * RY, NP = 5, R = 6;
+    static constexpr size_t BYTES = size_t(R) * NP * RP * sizeof(float);
+};
+
+// S8 and S10 for the pairwise collision: b_derivs on pairs of x-neighbouring sites, without A and B (see
+// b_collide_pair), 76 instead of 104 bytes written per site.  Packed FP32x2 arithmetic on 64-bit words;
+// u and rho - rho0 come by cp.async, each thread completing the words that it copied; p and the products
+// p u_b u_c are formed once per word of each stencil (x: three words instead of four points per site).
+// 522 -> 384 us at 256^3, 90 -> 67 us at 128^3 (64-wide tiles 413 and 73 us: their halo costs more than the
+// longer rows give).  Three CTAs of 128 threads per SM (138 registers, 52 KB of shared memory each).
+static __device__ __forceinline__ void b_derivs_pair(const DevSim& p, const Blk bid)
+{
+    using AL = AuxLayout<3>;
+    using DP = PairDerivsPlan;
+    constexpr int TX = DP::TX, TY = DP::TY, NT = DP::NT, RX = DP::RX, RP = DP::RP, NP = DP::NP, R = DP::R;
+    constexpr int HZ = 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* sr = reinterpret_cast<float*>(smem_raw);  // [R][NP][RY][RX]
+    const int tid = threadIdx.x;
+    const int x0 = bid.x * TX, y0 = bid.y * TY;
+    const int z0 = bid.z * p.zb[TK_DERIVS], z1 = min(z0 + p.zb[TK_DERIVS], p.nz);
+    const int NPL = p.nx * p.ny;
+    const float* drho = cp<float>(p.rho);
+    const float* uu = cp<float>(p.uit[0][p.us[0].cur]);  // S8: the converged u
+    const Phys<float>& q = p.pf;
+    constexpr int NG = RP / 2, MG = (NG + NT - 1) / NT;
+    int goff[MG];
+#pragma unroll
+    for (int m = 0; m < MG; ++m) {
+        const int t = tid + m * NT, gx = t % (RX / 2) * 2, gy = t / (RX / 2);
+        goff[m] = t < NG ? wrapm(x0 - 2 + gx, p.nx) + p.nx * wrapm(y0 - 2 + gy, p.ny) : 0;
+    }
+    auto fetch = [&](int zl, int sl) {
+        const int base = wrapc(zl, p.nz) * NPL;
+        float* dst = sr + sl * NP * RP;
+#pragma unroll
+        for (int m = 0; m < MG; ++m) {
+            const int t = tid + m * NT;
+            if (t < NG) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) cp_async<8>(dst + a * RP + t * 2, uu + a * p.N + (base + goff[m]));
+                cp_async<8>(dst + 3 * RP + t * 2, drho + (base + goff[m]));
+            }
+        }
+    };
+    const int ix = tid % (TX / 2) * 2, iy = tid / (TX / 2);
+    const int gx = x0 + ix, gy = y0 + iy;
+    const bool in = gx < p.nx && gy < p.ny;
+    const int sxy = gx + p.nx * gy;
+    int sl = (z0 - HZ + 8 * R) % R;  // ring slot of plane zl (z0 - HZ >= -2)
+    fetch(z0 - HZ, sl);
+    cp_async_commit();
+    for (int zl = z0 - HZ; zl < z1 + HZ; ++zl) {
+        const int zc = zl - HZ;
+        const bool act = zc >= z0 && in;
+        const int s = act ? sxy + NPL * zc : 0;
+        float2 j0[3] = {both(0.f), both(0.f), both(0.f)};  // own j0', before the barrier: the latency overlaps the wait
+        if (act) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) j0[a] = *reinterpret_cast<const float2*>(plane<float>(p.j0pp, a) + s);
+        }
+        cp_async_wait<0>();
+        {  // c_s^2 - c_s^2(rho0) at the words this thread copied
+            float* w = sr + sl * NP * RP;
+#pragma unroll
+            for (int m = 0; m < MG; ++m) {
+                const int t = tid + m * NT;
+                if (t < NG) {
+                    const float2 d = ld2<float>(w + 3 * RP + t * 2);
+                    *reinterpret_cast<float2*>(w + 4 * RP + t * 2) = cs2_delta2(p, d);
+                }
+            }
+        }
+        __syncthreads();
+        const int sn = sl + 1 == R ? 0 : sl + 1;  // held plane zl - 5, which only the previous pass read
+        if (zl + 1 < z1 + HZ) fetch(zl + 1, sn);
+        cp_async_commit();
+        if (zc + 1 >= z0 && zc + 1 < z1 && in) {  // own j0' of the next plane into L2
+#pragma unroll
+            for (int a = 0; a < 3; ++a) prefetch_l2(plane<float>(p.j0pp, a) + (sxy + NPL * (zc + 1)));
+        }
+        if (act) {
+            const float* pl[5];  // the pair's word in the planes zc - 2 .. zc + 2
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                const int b = 4 - k, t = sl >= b ? sl - b : sl - b + R;
+                pl[k] = sr + t * NP * RP + (iy + 2) * RX + ix + 2;
+            }
+            const float2 rho0 = both(q.rho0), cs0 = both(q.cs0), p0 = both(q.rho0 * q.cs0);
+            // the fields of one word: u, rho u_a (a the stencil's direction), p - p(rho0), p/rho - c_s^2(rho0), p u_b u_c
+            struct Word {
+                float2 u[3], ru, dp, dpr, puu[6];
+            };
+            auto word = [&](const float* g, int a) {
+                Word w;
+#pragma unroll
+                for (int b = 0; b < 3; ++b) w.u[b] = ld2<float>(g + b * RP);
+                const float2 d = ld2<float>(g + 3 * RP);
+                w.dpr = ld2<float>(g + 4 * RP);
+                w.ru = mul2(add2(rho0, d), w.u[a]);
+                w.dp = fma2(d, add2(cs0, w.dpr), mul2(rho0, w.dpr));
+                const float2 pf = add2(p0, w.dp);
+                const float2 pu[3] = {mul2(pf, w.u[0]), mul2(pf, w.u[1]), mul2(pf, w.u[2])};
+#pragma unroll
+                for (int b = 0; b < 3; ++b)
+#pragma unroll
+                    for (int c = b; c < 3; ++c) w.puu[sym2<3>(b, c)] = mul2(pu[b], w.u[c]);
+                return w;
+            };
+            float2 du[3][3], dp[3], dpr[3], dpuu[3][6], divj = both(0.f);
+            float2 rs, u[3];  // of the pair itself
+            auto deriv = [&](int a, auto d) {  // every derivative along a, d(member) of the loaded words
+#pragma unroll
+                for (int b = 0; b < 3; ++b) du[a][b] = d([b](const Word& w) { return w.u[b]; });
+                divj = add2(divj, d([](const Word& w) { return w.ru; }));
+                dp[a] = d([](const Word& w) { return w.dp; });
+                dpr[a] = d([](const Word& w) { return w.dpr; });
+#pragma unroll
+                for (int k = 0; k < 6; ++k) dpuu[a][k] = d([k](const Word& w) { return w.puu[k]; });
+            };
+            {
+                const float* g = pl[2];
+                const Word m = word(g - 2, 0), c = word(g, 0), n = word(g + 2, 0);
+                deriv(0, [&](auto get) { return d1x2(get(m), get(c), get(n)); });
+#pragma unroll
+                for (int a = 0; a < 3; ++a) u[a] = c.u[a];
+                rs = add2(rho0, ld2<float>(g + 3 * RP));
+            }
+            {
+                const float* g = pl[2];
+                const Word a = word(g - 2 * RX, 1), b = word(g - RX, 1), c = word(g + RX, 1), d = word(g + 2 * RX, 1);
+                deriv(1, [&](auto get) { return d1v2(get(a), get(b), get(c), get(d)); });
+            }
+            {
+                const Word a = word(pl[0], 2), b = word(pl[1], 2), c = word(pl[3], 2), d = word(pl[4], 2);
+                deriv(2, [&](auto get) { return d1v2(get(a), get(b), get(c), get(d)); });
+            }
+            // derivs_tail's formulas on both sites
+            float2 Pp, DPp, PMp, RPPp;
+            eos2(p, rs, Pp, DPp, PMp, RPPp);
+            auto out = [&](int c, float2 v) { *reinterpret_cast<float2*>(auxp<float>(p, c) + s) = v; };
+            const float2 divu = add2(add2(du[0][0], du[1][1]), du[2][2]);
+            const float2 irs = make_float2(1.f / rs.x, 1.f / rs.y);
+            const float2 kd = mul2(both(-q.k2), mul2(DPp, divj)), kr = mul2(mul2(both(q.k2), RPPp), mul2(divu, divj));
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = a; b < 3; ++b) {
+                    const float2 sd = add2(du[a][b], du[b][a]);
+                    out(AL::SIGL + sym2<3>(a, b), a == b ? fma2(kd, sd, kr) : mul2(kd, sd));
+                }
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+                out(AL::C + b, fma2(u[2], du[2][b], fma2(u[1], du[1][b], fma2(u[0], du[0][b], mul2(dp[b], irs)))));
+            float2 jt[3], Y[3];  // cj j~, and k3 [p d_c(p/rho) + (p - rho p') u_c div u]: the delta_ab terms of Xi'
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                jt[a] = mul2(both(q.cj), fma2(rs, u[a], mul2(both(-1.f), j0[a])));  // j~ = rho u - j0' (S8)
+                Y[a] = fma2(Pp, dpr[a], mul2(PMp, mul2(u[a], divu)));
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = a; b < 3; ++b)
+#pragma unroll
+                    for (int c = b; c < 3; ++c) {
+                        float2 v = add2(add2(dpuu[c][sym2<3>(a, b)], dpuu[b][sym2<3>(a, c)]), dpuu[a][sym2<3>(b, c)]);
+                        float2 j = both(0.f);
+                        if (a == b) { v = add2(v, Y[c]); j = add2(j, jt[c]); }
+                        if (a == c) { v = add2(v, Y[b]); j = add2(j, jt[b]); }
+                        if (b == c) { v = add2(v, Y[a]); j = add2(j, jt[a]); }
+                        out(AL::XI + sym3<3>(a, b, c), fma2(both(q.k3), v, j));
+                    }
+        }
+        sl = sn;
+    }
+}
+static __global__ void __launch_bounds__(PairDerivsPlan::NT, 3) k_derivs_pair(DevSim p)
+{
+    b_derivs_pair(p, launch_blk());
+}
+
+// ---------------------------------------------------------------------------
 // Batched forms of the step kernels.  A persistent grid walks the work list of every
 // simulation in the table: pass `item` is block (or tile) item - start[k] of slot k.  Slots
 // that do not take this step, and in the u-solve those whose solve has stopped, are skipped.
@@ -2142,21 +2785,21 @@ __global__ void __launch_bounds__(256, 3) kb_moments(const DevSim* sims, const B
     }
 }
 
-// tile coordinates of tile b of slot k
-__device__ __forceinline__ Blk batch_tile(const BatchWork* w, int k, int b)
+// tile coordinates of tile b of slot k of one tiled kernel
+__device__ __forceinline__ Blk batch_tile(const BatchWork* w, int kernel, int k, int b)
 {
-    const int gx = w->tgx[k], gy = w->tgy[k];
+    const int gx = w->tgx[kernel][k], gy = w->tgy[kernel][k];
     return Blk{b % gx, (b / gx) % gy, b / (gx * gy)};
 }
 
 template <int LAT, typename T, typename U>
 __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS) kb_force(const DevSim* sims, const BatchWork* w, int pair)
 {
-    const int n = w->nslot, total = w->tstart[n];
+    const int n = w->nslot, total = w->tstart[TK_FORCE][n];
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const int k = batch_slot(w->tstart, n, item);
+        const int k = batch_slot(w->tstart[TK_FORCE], n, item);
         if (!w->live[k]) continue;
-        b_force<LAT, T, U>(sims[k], pair, batch_tile(w, k, item - w->tstart[k]));
+        b_force<LAT, T, U>(sims[k], pair, batch_tile(w, TK_FORCE, k, item - w->tstart[TK_FORCE][k]));
         __syncthreads();
     }
 }
@@ -2171,11 +2814,11 @@ template <int LAT, typename T, typename U>
 __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, sizeof(U) == 4 ? 2 : 1)
     kb_sweep(const DevSim* sims, const BatchWork* w, int pair)
 {
-    const int n = w->nslot, total = w->tstart[n];
+    const int n = w->nslot, total = w->tstart[TK_SWEEP][n];
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const int k = batch_slot(w->tstart, n, item);
+        const int k = batch_slot(w->tstart[TK_SWEEP], n, item);
         if (!w->live[k] || !sims[k].us[pair].running) continue;
-        b_sweep<LAT, T, U, false>(sims[k], pair, batch_tile(w, k, item - w->tstart[k]));
+        b_sweep<LAT, T, U, false>(sims[k], pair, batch_tile(w, TK_SWEEP, k, item - w->tstart[TK_SWEEP][k]));
         __syncthreads();
     }
 }
@@ -2193,11 +2836,11 @@ static __global__ void kb_us_ctl(const DevSim* sims, const BatchWork* w, int pai
 template <int LAT, typename T, typename U>
 __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, 2) kb_derivs(const DevSim* sims, const BatchWork* w)
 {
-    const int n = w->nslot, total = w->tstart[n];
+    const int n = w->nslot, total = w->tstart[TK_DERIVS][n];
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const int k = batch_slot(w->tstart, n, item);
+        const int k = batch_slot(w->tstart[TK_DERIVS], n, item);
         if (!w->live[k]) continue;
-        b_derivs<LAT, T, U>(sims[k], batch_tile(w, k, item - w->tstart[k]));
+        b_derivs<LAT, T, U>(sims[k], batch_tile(w, TK_DERIVS, k, item - w->tstart[TK_DERIVS][k]));
         __syncthreads();
     }
 }
@@ -2205,11 +2848,34 @@ __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, 2) kb_derivs(const
 template <int LAT, typename T, int S, typename U, bool READ>
 __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, 2) kb_collide(const DevSim* sims, const BatchWork* w)
 {
-    const int n = w->nslot, total = w->tstart[n];
+    const int n = w->nslot, total = w->tstart[TK_COLLIDE][n];
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const int k = batch_slot(w->tstart, n, item);
+        const int k = batch_slot(w->tstart[TK_COLLIDE], n, item);
         if (!w->live[k]) continue;
-        b_collide<LAT, T, S, U, READ>(sims[k], w->src[k], batch_tile(w, k, item - w->tstart[k]));
+        b_collide<LAT, T, S, U, READ>(sims[k], w->src[k], batch_tile(w, TK_COLLIDE, k, item - w->tstart[TK_COLLIDE][k]));
+        __syncthreads();
+    }
+}
+
+static __global__ void __launch_bounds__(PairDerivsPlan::NT, 3) kb_derivs_pair(const DevSim* sims, const BatchWork* w)
+{
+    const int n = w->nslot, total = w->tstart[TK_DERIVS][n];
+    for (int item = blockIdx.x; item < total; item += gridDim.x) {
+        const int k = batch_slot(w->tstart[TK_DERIVS], n, item);
+        if (!w->live[k]) continue;
+        b_derivs_pair(sims[k], batch_tile(w, TK_DERIVS, k, item - w->tstart[TK_DERIVS][k]));
+        __syncthreads();
+    }
+}
+
+template <int S, bool READ, int W>
+__global__ void __launch_bounds__(PairCollidePlan<W>::NT, 2) kb_collide_pair(const DevSim* sims, const BatchWork* w)
+{
+    const int n = w->nslot, total = w->tstart[TK_COLLIDE][n];
+    for (int item = blockIdx.x; item < total; item += gridDim.x) {
+        const int k = batch_slot(w->tstart[TK_COLLIDE], n, item);
+        if (!w->live[k]) continue;
+        b_collide_pair<S, READ, W>(sims[k], w->src[k], batch_tile(w, TK_COLLIDE, k, item - w->tstart[TK_COLLIDE][k]));
         __syncthreads();
     }
 }
@@ -2431,6 +3097,26 @@ static __global__ void k_red_final(DevSim p, const double* part, int nparts, dou
 // ---------------------------------------------------------------------------
 // Kernel table of one combination
 // ---------------------------------------------------------------------------
+// Whether the derivative and collision kernels have their form on pairs of sites: 3D, FP32 deviations
+// from w_i(rho0) rho0 (the default of the workloads) and FP32 sweeps.  The pairwise forms round in another
+// order; with n_i itself in FP32, and with the 16-bit storages, such differences decide how stored
+// populations round and grow to the storage's own error, so those keep the forms they had, to the bit.
+template <int LAT, typename T, int S, typename U>
+constexpr bool kPairCollide = Lat<LAT>::D == 3 && sizeof(T) == 4 && sizeof(U) == 4 && S == ST_F32_DEV;
+
+// The collision on pairs of sites with tiles W wide.
+template <int S, int W>
+PairCollide pair_collide(bool read_pops)
+{
+    PairCollide t;
+    t.collide = read_pops ? (const void*)k_collide_pair<S, true, W> : (const void*)k_collide_pair<S, false, W>;
+    t.kb_collide = read_pops ? (const void*)kb_collide_pair<S, true, W> : (const void*)kb_collide_pair<S, false, W>;
+    t.tile = TileShape{PairCollidePlan<W>::TX, PairCollidePlan<W>::TY, PairCollidePlan<W>::NT};
+    t.smem = PairCollidePlan<W>::BYTES;
+    for (const void* f : {t.collide, t.kb_collide}) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem));
+    return t;
+}
+
 template <int LAT, typename T, int S, typename U>
 KernelTable make_table(bool read_pops)
 {
@@ -2463,9 +3149,7 @@ KernelTable make_table(bool read_pops)
     t.kb_step_end = (const void*)kb_step_end;
     t.block = 256;
     using TL = Tile<Lat<LAT>::D>;
-    t.tile[0] = TL::TX;
-    t.tile[1] = TL::TY;
-    t.tile_threads = TL::THREADS;
+    for (TileShape& ts : t.tile) ts = TileShape{TL::TX, TL::TY, TL::THREADS};
     constexpr int D = Lat<LAT>::D;
     t.smem_sweep = SweepPlan<D, T, U>::BYTES;
     t.sweep_box[0] = SweepPlan<D, T, U>::UX;
@@ -2478,6 +3162,16 @@ KernelTable make_table(bool read_pops)
     if (t.sweep_tma) cudaFuncSetAttribute(t.sweep_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_sweep));
     cudaFuncSetAttribute(t.derivs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_derivs));
     cudaFuncSetAttribute(t.collide, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_collide));
+    if constexpr (kPairCollide<LAT, T, S, U>) {
+        t.pair_collide[0] = pair_collide<S, 32>(read_pops);
+        t.pair_collide[1] = pair_collide<S, 64>(read_pops);
+        t.pair_derivs = (const void*)k_derivs_pair;
+        t.kb_pair_derivs = (const void*)kb_derivs_pair;
+        t.tile_pair_derivs = TileShape{PairDerivsPlan::TX, PairDerivsPlan::TY, PairDerivsPlan::NT};
+        t.smem_pair_derivs = PairDerivsPlan::BYTES;
+        for (const void* f : {t.pair_derivs, t.kb_pair_derivs})
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_pair_derivs));
+    }
     cudaFuncSetAttribute(t.kb_force, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_force));
     cudaFuncSetAttribute(t.kb_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_sweep));
     cudaFuncSetAttribute(t.kb_derivs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_derivs));
