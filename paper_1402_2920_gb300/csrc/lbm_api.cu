@@ -53,7 +53,7 @@ struct lbm_sim {
     int64_t steps = 0;
     std::vector<void*> allocs;
     double* red_part = nullptr;
-    double* red_out = nullptr;
+    HostView* view = nullptr;  // the device block that DevSim::us and DevSim::status point into
     Graphs one[2], two[2];
     bool graphs = false;  // the step graphs are built on the first lbm_step
 };
@@ -265,8 +265,8 @@ int add_step(lbm_sim* s, cudaGraph_t g, cudaGraphNode_t dep, int src, cudaGraphN
     DevSim& dv = s->dev;
     const int B = s->kt.block;
     const int G = nblocks(dv.N, B);
-    int pair = 0, one = 1;
-    cudaGraphNode_t n1, n2, n3, nc, n5, n6;
+    int pair = 0, mode = SWEEP_IN_GRAPH;
+    cudaGraphNode_t n1, n2[2], nc, n5, n6;
     const cudaGraphNode_t* d0 = dep ? &dep : nullptr;
     size_t nd0 = dep ? 1 : 0;
     {
@@ -276,11 +276,11 @@ int add_step(lbm_sim* s, cudaGraph_t g, cudaGraphNode_t dep, int src, cudaGraphN
     const TileShape* ts = s->kt.tile;
     {
         void* a[] = {&dv, &pair};
-        LBM_CK(add_kernel(g, &n2, s->kt.force, tile_grid(s, TK_FORCE), ts[TK_FORCE].threads, a, &n1, 1, s->kt.smem_force));
+        LBM_CK(add_kernel(g, &n2[0], s->kt.force, tile_grid(s, TK_FORCE), ts[TK_FORCE].threads, a, &n1, 1, s->kt.smem_force));
     }
-    {
+    {  // beside the force kernel: the solve's start needs the density range alone
         void* a[] = {&dv, &pair};
-        LBM_CK(add_kernel(g, &n3, s->kt.us_begin, dim3(1), 32, a, &n2, 1));
+        LBM_CK(add_kernel(g, &n2[1], s->kt.us_begin, dim3(1), 32, a, &n1, 1));
     }
     cudaGraphConditionalHandle h;
     LBM_CK(cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault));
@@ -289,14 +289,15 @@ int add_step(lbm_sim* s, cudaGraph_t g, cudaGraphNode_t dep, int src, cudaGraphN
     cp.conditional.handle = h;
     cp.conditional.type = cudaGraphCondTypeWhile;
     cp.conditional.size = 1;
-    LBM_CK(cudaGraphAddNode(&nc, g, &n3, nullptr, 1, &cp));
+    LBM_CK(cudaGraphAddNode(&nc, g, n2, nullptr, 2, &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     {
-        cudaGraphNode_t b1, b3;
-        void* a1[] = {&dv, &pair};
-        LBM_CK(add_kernel(body, &b1, s->sweep, tile_grid(s, TK_SWEEP), ts[TK_SWEEP].threads, a1, nullptr, 0, s->kt.smem_sweep));
-        void* a3[] = {&dv, &pair, &h, &one};
-        LBM_CK(add_kernel(body, &b3, s->kt.us_ctl, dim3(1), 1, a3, &b1, 1));
+        cudaGraphNode_t b1, b2;
+        void* a1[] = {&dv, &pair, &mode};
+        LBM_CK(add_kernel(body, &b1, s->sweep, tile_grid(s, TK_SWEEP), ts[TK_SWEEP].threads, a1, nullptr, 0,
+                          s->kt.smem_sweep));
+        void* a2[] = {&dv, &pair, &h, &mode};
+        LBM_CK(add_kernel(body, &b2, s->kt.us_ctl, dim3(1), 1, a2, &b1, 1));
     }
     {
         void* a[] = {&dv};
@@ -360,17 +361,18 @@ cudaError_t launch_tiled(const lbm_sim* s, TiledKernel k, A... args)
     return cudaLaunchKernel(fn[k], tile_grid(s, k), dim3(s->kt.tile[k].threads), a, smem[k], s->stream);
 }
 
-int read_status(lbm_sim* s, int* bits)
+// Everything issued so far is done, and the block is in *v.
+int read_view(lbm_sim* s, HostView* v)
 {
-    int st = 0;
-    LBM_CK(cudaMemcpyAsync(&st, s->dev.status, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    LBM_CK(cudaMemcpyAsync(v, s->view, sizeof(HostView), cudaMemcpyDeviceToHost, s->stream));
     LBM_CK(cudaStreamSynchronize(s->stream));
-    if (st) {
-        const int z = 0;
-        LBM_CK(cudaMemcpyAsync(s->dev.status, &z, sizeof(int), cudaMemcpyHostToDevice, s->stream));
-        LBM_CK(cudaStreamSynchronize(s->stream));
-    }
-    *bits = st;
+    return LBM_OK;
+}
+int clear_status(lbm_sim* s, int bits)
+{
+    if (!bits) return LBM_OK;
+    LBM_CK(cudaMemsetAsync(s->dev.status, 0, sizeof(int), s->stream));
+    LBM_CK(cudaStreamSynchronize(s->stream));
     return LBM_OK;
 }
 
@@ -446,21 +448,12 @@ void setup_sweep_maps(lbm_sim* s)
     if (ok) s->sweep = s->kt.sweep_tma;
 }
 
+// The u iterates need no reset: each solve's force kernel writes the one that its first sweep reads.
 int reset_usolve(lbm_sim* s)
 {
-    UsolveState z[2];
-    std::memset(z, 0, sizeof(z));
-    LBM_CK(cudaMemcpyAsync(s->dev.us, z, sizeof(z), cudaMemcpyHostToDevice, s->stream));
-    std::vector<unsigned> rg(4 * kRangeSlots);
-    for (int k = 0; k < 4 * kRangeSlots; ++k) rg[k] = ((k / kRangeSlots) % 2 == 0) ? 0x7f7fffffu : 0u;
-    LBM_CK(cudaMemcpyAsync(s->dev.range, rg.data(), rg.size() * sizeof(unsigned), cudaMemcpyHostToDevice, s->stream));
-    LBM_CK(cudaStreamSynchronize(s->stream));  // rg lives on this stack
+    LBM_CK(launch(s, s->kt.reset, 1, 256, s->dev));
     const size_t jbytes = 3 * size_t(s->dev.N) * s->kt.usize;
-    for (int pr = 0; pr < 2; ++pr)
-        for (int b = 0; b < 2; ++b) LBM_CK(cudaMemsetAsync(s->dev.uit[pr][b], 0, jbytes, s->stream));
     LBM_CK(cudaMemsetAsync(s->dev.jt_warm, 0, warm_buffers(s->dev) * jbytes, s->stream));
-    const int zi = 0;
-    LBM_CK(cudaMemcpyAsync(s->dev.status, &zi, sizeof(int), cudaMemcpyHostToDevice, s->stream));
     return LBM_OK;
 }
 
@@ -561,24 +554,29 @@ void choose_zb(lbm_sim* s)
     }
 }
 
-// S1-S8 on the current populations with the scratch j~ pair; host-driven loop.
-int run_fields(lbm_sim* s)
+// S1-S8 on the current populations with the scratch j~ pair, and the fields to device memory.  The sweeps are
+// launched kAhead at a time, the fields' kernel behind them: sweeps that come after the solve has stopped
+// return at once, and one copy tells whether it has.  (One sweep and one copy in turn left the device idle
+// for the host's round trip at each sweep.)
+int run_fields(lbm_sim* s, double* rho, double* u, HostView* v)
 {
+    constexpr int kAhead = 4;
     DevSim& dv = s->dev;
     const int B = s->kt.block, G = nblocks(dv.N, B);
-    const int pair = 1;
+    const int pair = 1, mode = SWEEP_BY_HOST;
+    const cudaGraphConditionalHandle h{};
     LBM_CK(launch_moments(s, dv, s->cur, pair));
     LBM_CK(launch_tiled(s, TK_FORCE, dv, pair));
     LBM_CK(launch(s, s->kt.us_begin, 1, 32, dv, pair));
-    cudaGraphConditionalHandle h{};
-    const int no = 0;
-    for (int it = 0; it < s->dev.maxit + 1; ++it) {
-        LBM_CK(launch_tiled(s, TK_SWEEP, dv, pair));
-        LBM_CK(launch(s, s->kt.us_ctl, 1, 1, dv, pair, h, no));
-        UsolveState u;
-        LBM_CK(cudaMemcpyAsync(&u, &dv.us[1], sizeof(u), cudaMemcpyDeviceToHost, s->stream));
-        LBM_CK(cudaStreamSynchronize(s->stream));
-        if (!u.running) break;  // the control kernel recorded a stop
+    for (int it = 0; it < dv.maxit + 1; it += kAhead) {
+        for (int k = 0; k < kAhead; ++k) {
+            LBM_CK(launch_tiled(s, TK_SWEEP, dv, pair, mode));
+            LBM_CK(launch(s, s->kt.us_ctl, 1, 1, dv, pair, h, mode));
+        }
+        LBM_CK(launch(s, s->kt.fields_out, G, B, dv, 1, rho, u));
+        const int rc = read_view(s, v);
+        if (rc) return rc;
+        if (!v->us[1].running) break;  // the control step recorded a stop
     }
     return LBM_OK;
 }
@@ -820,19 +818,19 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
                 dv.jwp[b][a] = static_cast<char*>(dv.jt_warm) + size_t((warm_buffers(dv) - 1) * b * 3 + a) * N * U;
         }
     }
-    void* usp = nullptr;
-    rc = rc ? rc : dev_alloc(s, &usp, 2 * sizeof(UsolveState));
-    dv.us = static_cast<UsolveState*>(usp);
+    void* vp = nullptr;
+    rc = rc ? rc : dev_alloc(s, &vp, sizeof(HostView));
+    s->view = static_cast<HostView*>(vp);
+    if (!rc) {
+        dv.us = s->view->us;
+        dv.status = &s->view->status;
+    }
     void* rgp = nullptr;
     rc = rc ? rc : dev_alloc(s, &rgp, 4 * kRangeSlots * sizeof(unsigned));
     dv.range = static_cast<unsigned*>(rgp);
-    void* stp = nullptr;
-    rc = rc ? rc : dev_alloc(s, &stp, 256);
-    dv.status = static_cast<int*>(stp);
     void* rp = nullptr;
-    rc = rc ? rc : dev_alloc(s, &rp, (kRedGrid * 4 + 8) * sizeof(double));
+    rc = rc ? rc : dev_alloc(s, &rp, kRedGrid * 4 * sizeof(double));
     s->red_part = static_cast<double*>(rp);
-    s->red_out = s->red_part + kRedGrid * 4;
     dv.red = s->red_part;
     if (rc) { lbm_destroy(s); return rc; }
     {  // vector (16-byte) copies of the tiled kernels need 16-byte aligned field arrays
@@ -854,7 +852,10 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
             return LBM_E_CUDA;
         }
     }
-    rc = reset_usolve(s);
+    for (int pr = 0; pr < 2; ++pr)
+        for (int b = 0; b < 2; ++b)
+            if (cudaMemsetAsync(dv.uit[pr][b], 0, 3 * N * U, s->stream) != cudaSuccess) rc = LBM_E_CUDA;
+    if (!rc) rc = reset_usolve(s);
     if (!rc && cudaStreamSynchronize(s->stream) != cudaSuccess) rc = LBM_E_CUDA;
     if (rc) { lbm_destroy(s); return rc; }
     *out = s;
@@ -895,6 +896,7 @@ int lbm_init(lbm_sim* s, const double* rho, const double* u, int on_device)
         double* p = tmp;
         tmp = nullptr;
         LBM_CK(cudaFreeAsync(p, s->stream));
+        LBM_CK(cudaStreamSynchronize(s->stream));  // the caller's host arrays are borrowed for the call only
     }
     return LBM_OK;
 }
@@ -915,14 +917,14 @@ int step_direct(lbm_sim* s)
 {
     DevSim& dv = s->dev;
     const int B = s->kt.block, G = nblocks(dv.N, B);
-    const int pair = 0, no = 0, src = s->cur;
-    cudaGraphConditionalHandle h{};
+    const int pair = 0, mode = SWEEP_BY_HOST, src = s->cur;
+    const cudaGraphConditionalHandle h{};
     LBM_CK(launch_moments(s, dv, src, pair));
     LBM_CK(launch_tiled(s, TK_FORCE, dv, pair));
     LBM_CK(launch(s, s->kt.us_begin, 1, 32, dv, pair));
     for (int it = 0; it < dv.maxit + 1; ++it) {
-        LBM_CK(launch_tiled(s, TK_SWEEP, dv, pair));
-        LBM_CK(launch(s, s->kt.us_ctl, 1, 1, dv, pair, h, no));
+        LBM_CK(launch_tiled(s, TK_SWEEP, dv, pair, mode));
+        LBM_CK(launch(s, s->kt.us_ctl, 1, 1, dv, pair, h, mode));
         UsolveState u;
         LBM_CK(cudaMemcpyAsync(&u, &dv.us[0], sizeof(u), cudaMemcpyDeviceToHost, s->stream));
         LBM_CK(cudaStreamSynchronize(s->stream));
@@ -981,21 +983,17 @@ int lbm_sync(lbm_sim* s)
 {
     if (!s) return LBM_E_INVALID_ARG;
     LBM_CK(cudaSetDevice(s->device));
-    LBM_CK(cudaStreamSynchronize(s->stream));
-    int bits = 0;
-    int rc = read_status(s, &bits);
-    if (rc) return rc;
-    return status_code(bits);
+    HostView v;
+    int rc = read_view(s, &v);
+    rc = rc ? rc : clear_status(s, v.status);
+    return rc ? rc : status_code(v.status);
 }
 
 int lbm_fields(lbm_sim* s, double* rho, double* u, int on_device)
 {
     if (!s) return LBM_E_INVALID_ARG;
     LBM_CK(cudaSetDevice(s->device));
-    int rc = run_fields(s);
-    if (rc) return rc;
     const size_t N = size_t(s->dev.N);
-    const int B = s->kt.block, G = nblocks(s->dev.N, B);
     double* drho = rho;
     double* du = u;
     double* tmp = nullptr;
@@ -1004,17 +1002,19 @@ int lbm_fields(lbm_sim* s, double* rho, double* u, int on_device)
         drho = rho ? tmp : nullptr;
         du = u ? tmp + N : nullptr;
     }
-    LBM_CK(launch(s, s->kt.fields_out, G, B, s->dev, 1, drho, du));
+    HostView v;
+    int rc = run_fields(s, drho, du, &v);
     if (tmp) {
-        if (rho) LBM_CK(cudaMemcpyAsync(rho, drho, N * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-        if (u) LBM_CK(cudaMemcpyAsync(u, du, s->d * N * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-        LBM_CK(cudaFreeAsync(tmp, s->stream));
+        if (!rc && rho && cudaMemcpyAsync(rho, drho, N * sizeof(double), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
+            rc = LBM_E_CUDA;
+        if (!rc && u && cudaMemcpyAsync(u, du, s->d * N * sizeof(double), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
+            rc = LBM_E_CUDA;
+        if (cudaFreeAsync(tmp, s->stream) != cudaSuccess && !rc) rc = LBM_E_CUDA;
+        if (!rc && cudaStreamSynchronize(s->stream) != cudaSuccess) rc = LBM_E_CUDA;
+        if (rc) (void)cudaGetLastError();
     }
-    LBM_CK(cudaStreamSynchronize(s->stream));
-    int bits = 0;
-    rc = read_status(s, &bits);
-    if (rc) return rc;
-    return status_code(bits);
+    rc = rc ? rc : clear_status(s, v.status);
+    return rc ? rc : status_code(v.status);
 }
 
 int lbm_populations(lbm_sim* s, double* out, int on_device)
@@ -1070,23 +1070,20 @@ int lbm_stats_get(lbm_sim* s, lbm_stats* out)
     if (!s || !out) return LBM_E_INVALID_ARG;
     LBM_CK(cudaSetDevice(s->device));
     LBM_CK(launch(s, s->kt.red_partial, kRedGrid, kRedBlock, s->dev, s->cur, s->red_part));
-    LBM_CK(launch(s, s->kt.red_final, 1, kRedBlock, s->dev, (const double*)s->red_part, kRedGrid, s->red_out));
-    double sums[4];
-    UsolveState u;
-    int st = 0;
-    LBM_CK(cudaMemcpyAsync(sums, s->red_out, sizeof(sums), cudaMemcpyDeviceToHost, s->stream));
-    LBM_CK(cudaMemcpyAsync(&u, &s->dev.us[0], sizeof(u), cudaMemcpyDeviceToHost, s->stream));
-    LBM_CK(cudaMemcpyAsync(&st, s->dev.status, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-    LBM_CK(cudaStreamSynchronize(s->stream));
-    out->mass = sums[0];
-    out->mom[0] = sums[1];
-    out->mom[1] = sums[2];
-    out->mom[2] = sums[3];
+    LBM_CK(launch(s, s->kt.red_final, 1, kRedBlock, s->dev, (const double*)s->red_part, kRedGrid, s->view->sums));
+    HostView v;
+    const int rc = read_view(s, &v);
+    if (rc) return rc;
+    const UsolveState& u = v.us[0];
+    out->mass = v.sums[0];
+    out->mom[0] = v.sums[1];
+    out->mom[1] = v.sums[2];
+    out->mom[2] = v.sums[3];
     out->steps = s->steps;
     out->usolve_iters_last = u.iters_last;
     out->usolve_iters_max = u.iters_max;
     out->usolve_resid = u.resid_last;
-    out->status = st;
+    out->status = v.status;
     out->usolve_sweeps_total = u.sweeps_total;
     out->usolve_tensor_copies = u.tma;
     return LBM_OK;
@@ -1111,6 +1108,7 @@ int lbm_profile(lbm_sim* s, int reps, double* ms_out, int n)
     LBM_CK(launch_moments(s, dv, src, pair));
     LBM_CK(launch_tiled(s, TK_FORCE, dv, pair));
     LBM_CK(launch(s, s->kt.us_begin, 1, 32, dv, pair));
+    const int alone = SWEEP_ALONE;
     int rc = LBM_OK;
     for (int k = 0; k < 5 && rc == LBM_OK; ++k) {
         for (int r = 0; r <= reps && rc == LBM_OK; ++r) {
@@ -1119,7 +1117,7 @@ int lbm_profile(lbm_sim* s, int reps, double* ms_out, int n)
             switch (k) {
             case 0: e = launch_moments(s, dv, src, pair); break;
             case 1: e = launch_tiled(s, TK_FORCE, dv, pair); break;
-            case 2: e = launch_tiled(s, TK_SWEEP, dv, pair); break;
+            case 2: e = launch_tiled(s, TK_SWEEP, dv, pair, alone); break;
             case 3: e = launch_tiled(s, TK_DERIVS, dv); break;
             case 4: e = launch_tiled(s, TK_COLLIDE, dv, src); break;
             }
@@ -1221,6 +1219,7 @@ int lbm_load(lbm_sim* s, const char* path)
     LBM_CK(cudaStreamSynchronize(s->stream));
     int rc = reset_usolve(s);
     if (rc) return rc;
+    LBM_CK(cudaStreamSynchronize(s->stream));  // the copies below do not go through the stream
     s->cur = 0;
     u0.cur = 0;
     u0.resid_bits = 0;

@@ -40,6 +40,13 @@ struct UsolveState {
     int opened;                     // 1: this solve (after it: the last one) opened with plain sweeps
 };
 
+// What the host reads back of a simulation: one device block, one copy.
+struct HostView {
+    UsolveState us[2];
+    double sums[4];  // conservation sums
+    int status;      // error bits
+};
+
 // planes ahead of the one in work whose per-site inputs the collision and derivative
 // kernels prefetch into L2 (measured at 256^3)
 constexpr int kCollideLead = 1;
@@ -63,6 +70,10 @@ enum TiledKernel { TK_FORCE = 0, TK_SWEEP, TK_DERIVS, TK_COLLIDE, kTiled };
 struct TileShape {
     int tx, ty, threads;
 };
+
+// How a sweep and its control step are launched: one by one by the host, several ahead, which do nothing once
+// the solve has stopped; in a graph, whose loop condition the control sets; or alone (kernel timing).
+enum SweepMode { SWEEP_BY_HOST = 0, SWEEP_IN_GRAPH = 1, SWEEP_ALONE = 2 };
 
 // slots of the density-range reduction (spread so that block atomics do not contend)
 constexpr int kRangeSlots = 64;
@@ -153,7 +164,7 @@ struct DevSim {
     // plane tables of the aux field (aux + c N) and of the 3-vector fields j0', f and the warm-start
     // j~ (field + a N), in the field's element type.  jwp[b]: warm-start buffer b.  The force kernel
     // starts the u-solve from jwp[wsel] (the newest j~) and, for warm = 2, jwp[wsel ^ 1] (the one
-    // before); the run's k_us_begin flips wsel, and the collision writes the new j~ over the older
+    // before); the run's control step flips wsel when the solve stops, and the collision writes the new j~ over the older
     // one.  With one buffer (warm < 2) both entries name it.
     void* auxp[26];
     void* j0pp[3];
@@ -197,11 +208,13 @@ struct KernelTable {
     const void* moments;      // (DevSim, int src, int pair)
     const void* force;        // (DevSim, int pair): also the u-solve's starting u
     const void* us_begin;     // (DevSim, int pair)
-    const void* sweep;        // (DevSim, int pair): one tiled u-solve sweep, planes copied per thread
+    const void* sweep;        // (DevSim, int pair, int SweepMode): one tiled u-solve sweep, planes copied
+                              // per thread
     const void* sweep_tma;    // the same with tensor-copy (TMA) plane loads (3D; nullptr in 2D)
-    const void* us_ctl;       // (DevSim, int pair, cudaGraphConditionalHandle, int use_cond)
+    const void* us_ctl;       // (DevSim, int pair, cudaGraphConditionalHandle, int SweepMode)
     const void* derivs;       // (DevSim)
     const void* collide;      // (DevSim, int src)
+    const void* reset;        // (DevSim): one block
     const void* init_eq;      // (DevSim, const double* rho, const double* u, int dst)
     const void* init_ref;     // (DevSim, const double* rho, int dst): local-reference storages only
     const void* pops_rho;     // (DevSim, const double* pops, double* rho): sum over i of FP64 populations

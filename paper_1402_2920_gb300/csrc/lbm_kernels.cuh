@@ -596,7 +596,6 @@ static __device__ void b_us_begin(const DevSim& p, int pair, int lane)
     if (lane != 0) return;
     g = fmin(0.95, 1.02 * g);
     u.gain = g;
-    if (pair == 0) u.wsel ^= 1;  // the run's collision writes this step's j~ over the older one
     u.cheb_delta = 0.5 * g;
     u.cheb_sigma = (1.0 - 0.5 * g) / (0.5 * g);
     u.iter = 0;
@@ -678,13 +677,17 @@ static __device__ bool b_us_ctl(const DevSim& p, int pair)
         u.iters_max = u.iter > u.iters_max ? u.iter : u.iters_max;
         u.converged = conv ? 1 : 0;
         u.running = 0;
+        if (pair == 0) u.wsel ^= 1;  // the run's collision writes this step's j~ over the older one
     }
     return stop;
 }
-static __global__ void k_us_ctl(DevSim p, int pair, cudaGraphConditionalHandle h, int use_cond)
+// (Run by the last CTA of the sweep, behind a ticket, the control step cost the small lattices 2 to 4 us a
+// sweep more than this launch, which the graph prepares while the sweep runs.)
+static __global__ void k_us_ctl(DevSim p, int pair, cudaGraphConditionalHandle h, int mode)
 {
+    if (!p.us[pair].running) return;  // launched ahead, and the solve has stopped
     const bool stop = b_us_ctl(p, pair);
-    if (use_cond) cudaGraphSetConditional(h, stop ? 0u : 1u);
+    if (mode == SWEEP_IN_GRAPH) cudaGraphSetConditional(h, stop ? 0u : 1u);
 }
 
 // ---------------------------------------------------------------------------
@@ -1538,8 +1541,9 @@ __device__ __forceinline__ void b_sweep(const DevSim& p, int pair, const Blk bid
     block_max2(dmax_d, double(jmax), &p.us[pair].resid_bits, &p.us[pair].jmax_bits);
 }
 template <int LAT, typename T, typename U, bool TMA>
-__global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, sizeof(U) == 4 ? 3 : 1) k_sweep(DevSim p, int pair)
+__global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, sizeof(U) == 4 ? 3 : 1) k_sweep(DevSim p, int pair, int mode)
 {
+    if (mode == SWEEP_BY_HOST && !p.us[pair].running) return;  // launched ahead, and the solve has stopped
     b_sweep<LAT, T, U, TMA>(p, pair, launch_blk());
 }
 
@@ -2880,6 +2884,15 @@ __global__ void __launch_bounds__(PairCollidePlan<W>::NT, 2) kb_collide_pair(con
     }
 }
 
+// The u-solve's state, density ranges and error bits before a first step (one block).
+static __global__ void k_reset(DevSim p)
+{
+    int* us = reinterpret_cast<int*>(p.us);
+    for (int k = threadIdx.x; k < int(2 * sizeof(UsolveState) / sizeof(int)); k += blockDim.x) us[k] = 0;
+    for (int k = threadIdx.x; k < 4 * kRangeSlots; k += blockDim.x) p.range[k] = (k / kRangeSlots) % 2 == 0 ? 0x7f7fffffu : 0u;
+    if (threadIdx.x == 0) *p.status = 0;
+}
+
 // ---------------------------------------------------------------------------
 // Initial condition, field and population transfer, conservation sums
 // ---------------------------------------------------------------------------
@@ -3170,11 +3183,12 @@ KernelTable make_table(bool read_pops)
     t.moments = (const void*)k_moments<LAT, T, S, U>;
     t.force = (const void*)k_force<LAT, T, U>;
     t.us_begin = (const void*)k_us_begin;
+    t.us_ctl = (const void*)k_us_ctl;
     t.sweep = (const void*)k_sweep<LAT, T, U, false>;
     t.sweep_tma = Lat<LAT>::D == 3 ? (const void*)k_sweep<LAT, T, U, true> : nullptr;
-    t.us_ctl = (const void*)k_us_ctl;
     t.derivs = (const void*)k_derivs<LAT, T, U>;
     t.collide = read_pops ? (const void*)k_collide<LAT, T, S, U, true> : (const void*)k_collide<LAT, T, S, U, false>;
+    t.reset = (const void*)k_reset;
     t.init_eq = (const void*)k_init_eq<LAT, T, S>;
     t.init_ref = Codec<S>::LOC ? (const void*)k_init_ref<LAT, T> : nullptr;
     t.pops_rho = (const void*)k_pops_rho<LAT>;
