@@ -296,7 +296,8 @@ def run_native(args):
     ms, clocks, sweeps, st = timed(sim, K, Wm)
     tensor_copies = st.usolve_tensor_copies  # 1: the sweeps' plane loads ran as tensor copies (TMA)
     mlups = whole_job_mlups(ws, N, K, ms / 1e3)
-    launches = 5 * K + 2 * sweeps  # moments, force, u-solve start, derivs, collide; sweep + control
+    # moments, force, u-solve start, derivs, collide; sweep + control (three of them in every step, idle or not)
+    launches = 5 * K + 2 * max(sweeps, 3 * K)
 
     # dominant kernel: average launch time from CUDA events on the simulation's stream
     prof = P.lbm_profile(sim.handle, reps=5)

@@ -1543,7 +1543,7 @@ __device__ __forceinline__ void b_sweep(const DevSim& p, int pair, const Blk bid
 template <int LAT, typename T, typename U, bool TMA>
 __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, sizeof(U) == 4 ? 3 : 1) k_sweep(DevSim p, int pair, int mode)
 {
-    if (mode == SWEEP_BY_HOST && !p.us[pair].running) return;  // launched ahead, and the solve has stopped
+    if (mode != SWEEP_ALONE && !p.us[pair].running) return;  // launched ahead, and the solve has stopped
     b_sweep<LAT, T, U, TMA>(p, pair, launch_blk());
 }
 
