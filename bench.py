@@ -85,23 +85,26 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(self.samples)}
 
 
-def _algorithmic_bytes(lattice, storage_bytes, read_pops, chebyshev=True):
+def _algorithmic_bytes(lattice, storage_bytes, read_pops, chebyshev=True, pairwise=False):
     """Bytes each kernel must move per site if every input and output is touched once (FP32 fields).
 
     The rest population of the deviation storages is a float pair (8 bytes) and the density
-    carries its float remainder rho_lo (4 bytes), both read once per step by the collision."""
+    carries its float remainder rho_lo (4 bytes), both read once per step by the collision.
+    pairwise: the kernels of the 3D FP32 deviations with nx even, which keep 19 aux fields (no A, B) and
+    a pressure pair that the force kernel writes and the sweep reads."""
     Q, d = (59, 3) if lattice == 1 else (21, 2)
-    naux = 26 if lattice == 1 else 13
+    naux = 19 if pairwise else 26 if lattice == 1 else 13
     f = 4
+    pm = 2 * f if pairwise else 0
     pops = (Q - 1) * storage_bytes + 8
     return {
         # read the populations, write rho - rho0, rho_lo and j0
         "moments": pops + (2 + d) * f,
         # read rho - rho0, j0 and the last two steps' j~ (the extrapolated start); write f, j0' and
         # the starting u
-        "force": f + 3 * d * f + 3 * d * f,
+        "force": f + 3 * d * f + 3 * d * f + pm,
         # read u, rho - rho0, j0'; write u (Chebyshev: read and write the update vector too)
-        "usolve_sweep": f + 3 * d * f + (2 * d * f if chebyshev else 0),
+        "usolve_sweep": f + 3 * d * f + (2 * d * f if chebyshev else 0) + pm,
         # read u, rho - rho0, j0'; write A, B, C, the local Sigma and Xi'
         "derivs": f + 2 * d * f + naux * f,
         # read A, B, C, Sigma_local, Xi', rho - rho0, rho_lo, u, j0', f; write j~ and the populations
@@ -304,7 +307,8 @@ def run_native(args):
     per_step = {k: v * (sweeps / K if k.startswith("usolve") else 1.0) for k, v in prof.items()}
     dom = max(per_step, key=per_step.get)
     sb = STORAGE_BYTES[args.storage]
-    alg = _algorithmic_bytes(case.lattice, sb, case.gamma != 0.0)
+    alg = _algorithmic_bytes(case.lattice, sb, case.gamma != 0.0,
+                             pairwise=storage == P.LBM_STORE_F32_DEV and case.dims[0] % 2 == 0)
     peak, peak_kind = _peaks()
     achieved = alg[dom] * N / (prof[dom] / 1e3) / 1e9
     step_gbs = 2 * 59 * sb * N / (ms / K / 1e3) / 1e9  # whole step against 2 Q s bytes per site

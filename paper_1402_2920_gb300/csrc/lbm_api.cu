@@ -421,8 +421,9 @@ EncodeTiledFn tensor_map_encoder()
 }
 
 // Tensor map of a field [ncomp][nz][ny][nx] (rank 3 when ncomp = 1) read in boxes of one plane of
-// box_x x box_y sites, out-of-range elements read as zero.
-bool encode_plane_map(CUtensorMap* m, void* base, int ncomp, size_t esize, const DevSim& dv, const int box[2])
+// box_x x box_y sites and box_comps components, out-of-range elements read as zero.
+bool encode_plane_map(CUtensorMap* m, void* base, int ncomp, size_t esize, const DevSim& dv, int box_x, int box_y,
+                      int box_comps)
 {
     const EncodeTiledFn enc = tensor_map_encoder();
     if (!enc || !base) return false;
@@ -430,7 +431,7 @@ bool encode_plane_map(CUtensorMap* m, void* base, int ncomp, size_t esize, const
     const cuuint64_t dims[4] = {cuuint64_t(dv.nx), cuuint64_t(dv.ny), cuuint64_t(dv.nz), cuuint64_t(ncomp)};
     const cuuint64_t strides[3] = {cuuint64_t(dv.nx) * esize, cuuint64_t(dv.nx) * cuuint64_t(dv.ny) * esize,
                                    cuuint64_t(dv.N) * esize};
-    const cuuint32_t boxd[4] = {cuuint32_t(box[0]), cuuint32_t(box[1]), 1, 1};
+    const cuuint32_t boxd[4] = {cuuint32_t(box_x), cuuint32_t(box_y), 1, cuuint32_t(box_comps)};
     const cuuint32_t es[4] = {1, 1, 1, 1};
     const CUresult r = enc(m, esize == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rank, base,
                            dims, strides, boxd, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -452,11 +453,13 @@ void setup_sweep_maps(lbm_sim* s)
     if ((sel && std::strcmp(sel, "cp_async") == 0) || !s->kt.sweep_tma) return;
     if (s->d != 3 || !dv.aligned16 || dv.nx % 4 != 0) return;
     SweepMaps m;
+    const int bx = s->kt.sweep_box[0], by = s->kt.sweep_box[1];
     bool ok = true;
     for (int pr = 0; pr < 2; ++pr)
         for (int b = 0; b < 2; ++b)
-            ok = ok && encode_plane_map(&m.u[pr][b], dv.uit[pr][b], 3, s->kt.usize, dv, s->kt.sweep_box);
-    ok = ok && encode_plane_map(&m.rho, dv.rho, 1, s->kt.tsize, dv, s->kt.sweep_box);
+            ok = ok && encode_plane_map(&m.u[pr][b], dv.uit[pr][b], 3, s->kt.usize, dv, bx, by, dv.pm ? 3 : 1);
+    ok = ok && (dv.pm ? encode_plane_map(&m.rho, dv.pm, 2, sizeof(float), dv, bx, s->kt.pm_rows, 2)
+                      : encode_plane_map(&m.rho, dv.rho, 1, s->kt.tsize, dv, bx, by, 1));
     void* dm = nullptr;
     ok = ok && dev_alloc(s, &dm, sizeof(SweepMaps)) == LBM_OK;
     ok = ok && cudaMemcpyAsync(dm, &m, sizeof(SweepMaps), cudaMemcpyHostToDevice, s->stream) == cudaSuccess &&
@@ -541,11 +544,17 @@ void choose_zb(lbm_sim* s)
                     {s->sweep, s->kt.smem_sweep, 6.0, {1.3, 1.65, 2.2, 2.9}, 16.6},
                     {s->kt.derivs, s->kt.smem_derivs, 1.5, {1.8, 2.2, 2.9, 3.9}, 31.0},
                     {s->kt.collide, s->kt.smem_collide, 0.5, {3.3, 6.6, 9.9, 13.2}, 60.0}};
+    auto set = [&](TiledKernel k, double halo, double l1, double l2, double l3, double l4) {
+        ks[k].halo = halo;
+        ks[k].l[0] = l1, ks[k].l[1] = l2, ks[k].l[2] = l3, ks[k].l[3] = l4;
+    };
+    if (s->kt.pm_rows) {  // b_sweep_pm, and the force kernel that writes its pressure pair
+        set(TK_FORCE, 2.0, 1.0, 1.35, 1.7, 2.1);
+        set(TK_SWEEP, 8.0, 0.95, 1.4, 1.7, 2.3);
+    }
     if (s->kt.derivs == s->kt.pair_derivs) {  // the kernels on pairs of sites
-        const double ld[RMAX] = {1.5, 2.0, 2.55, 3.4}, lc[RMAX] = {2.75, 5.0, 7.5, 10.0};
-        for (int m = 0; m < RMAX; ++m) ks[TK_DERIVS].l[m] = ld[m], ks[TK_COLLIDE].l[m] = lc[m];
-        ks[TK_DERIVS].halo = 1.3;
-        ks[TK_COLLIDE].halo = 0.3;
+        set(TK_DERIVS, 1.3, 1.5, 2.0, 2.55, 3.4);
+        set(TK_COLLIDE, 0.3, 2.75, 5.0, 7.5, 10.0);
     }
     for (int q = 0; q < kTiled; ++q) {
         Kern& k = ks[q];
@@ -811,6 +820,11 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
     if (s->kt.exact) rc = rc ? rc : dev_alloc(s, &dv.rho_lo, N * sizeof(float));
     rc = rc ? rc : dev_alloc(s, &dv.rho, N * T);
     rc = rc ? rc : dev_alloc(s, &dv.j0p, 3 * N * T);
+    if (s->kt.pm_rows) {
+        void* w = nullptr;
+        rc = rc ? rc : dev_alloc(s, &w, 2 * N * sizeof(float));
+        dv.pm = static_cast<float*>(w);
+    }
     rc = rc ? rc : dev_alloc(s, &dv.f, 3 * N * T);
     for (int pr = 0; pr < 2; ++pr)
         for (int b = 0; b < 2; ++b) rc = rc ? rc : dev_alloc(s, &dv.uit[pr][b], 3 * N * U);

@@ -127,6 +127,8 @@ struct DevSim {
     void* jt_warm;        // U [nw][3][N]: j~ = rho u - j0' of the last step, the warm start (Sec. IX),
                           // and with the extrapolated start (warm = 2) that of the step before
     void* aux;            // T [26][N]: A, B_ab, C_a, the local part of Sigma_ab, Xi'_abc
+    float* pm;            // [2][N]: -p/27 and -(p - rho p')/27 of every site, left by the force kernel for b_sweep_pm
+                          // (3D FP32 deviations with FP32 sweeps; else null)
     float* wref[2];       // [NSHELL][N] per population buffer (local-reference storages): w_k(c_s^2(rho)) rho
                           // of every site at the collision that sent the populations in that buffer
     UsolveState* us;      // [2]: pair 0 and pair 1
@@ -176,6 +178,7 @@ struct DevSim {
 
 // The sweep's tensor maps: the u iterates uit[pair][buffer] as {nx, ny, nz, 3} and rho - rho0
 // as {nx, ny, nz}, each loaded in boxes of one plane: the sweep's tile with its in-plane halo of 4.
+// With b_sweep_pm a box holds all components, and `rho` is the pressure pair DevSim::pm.
 struct SweepMaps {
     CUtensorMap u[2][2];
     CUtensorMap rho;
@@ -244,6 +247,7 @@ struct KernelTable {
     size_t tsize, usize, ssize;  // bytes of T, U and the storage type
     size_t rsize;                // bytes of a rest-plane element (0: no separate plane)
     int sweep_box[2];            // in-plane box of the sweep's plane loads (tile plus halo 4)
+    int pm_rows;                 // rows of the pressure pair's box (b_sweep_pm; 0: the sweep has none)
     bool exact;                  // float-pair density bookkeeping (rho_lo is used)
     bool local_ref;              // the storage is relative to the sender's w_k rho (DevSim::wref)
 };

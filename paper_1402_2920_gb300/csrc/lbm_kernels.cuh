@@ -1589,6 +1589,294 @@ __device__ __forceinline__ float2 d1x2(float2 xm, float2 xc, float2 xp)
     return fma2(both(float(2.0 / 3.0)), make_float2(xc.y - xm.y, xp.x - xc.x),
                 mul2(both(-float(1.0 / 12.0)), sub2(xp, xm)));
 }
+// maximum that keeps a NaN
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+// 3/2 of the Sec. IV.B first derivative: (p1 - m1) - (1/8)(p2 - m2)
+__device__ __forceinline__ float d1s(float m2, float m1, float p1, float p2) { return __fmaf_rn(-0.125f, p2 - m2, p1 - m1); }
+__device__ __forceinline__ float2 d1s2(float2 m2, float2 m1, float2 p1, float2 p2)
+{
+    return fma2(both(-0.125f), sub2(p2, m2), sub2(p1, m1));
+}
+__device__ __forceinline__ float2 d1sx2(float2 xm, float2 xc, float2 xp)  // along x, see d1x2
+{
+    return fma2(both(-0.125f), sub2(xp, xm), make_float2(xc.y - xm.y, xp.x - xc.x));
+}
+
+// Shared memory of b_sweep_pm: a ring of u (halo 4; five planes of the stencil and one in flight), two planes
+// of the pressure pair (rows with halo 2; one in use, one in flight) and two q planes.
+struct SweepPmPlan {
+    static constexpr int TX = 32, TY = 8, NT = TX * TY;
+    static constexpr int UX = TX + 8, UY = TY + 8, UP = UX * UY;
+    static constexpr int QX = TX + 4, QY = TY + 4, QP = QX * QY, NQ = 6, PP = UX * QY;
+    static constexpr int R = 6;
+    static constexpr size_t OFF_P = size_t(R) * 3 * UP * sizeof(float);             // 128-byte multiples: tensor copies
+    static constexpr size_t OFF_Q = OFF_P + size_t(2) * 2 * PP * sizeof(float);
+    static constexpr size_t BYTES = OFF_Q + size_t(2) * NQ * QP * sizeof(float) + 128;
+    static_assert(OFF_P % 128 == 0 && (3 * UP * sizeof(float)) % 128 == 0 && (2 * PP * sizeof(float)) % 128 == 0, "");
+};
+
+// S3-S6 fused for the 3D FP32-deviation storage: b_sweep's march and stages (see there), leaner.
+//   - The force kernel leaves -p/27 and -(p - rho p')/27 of every site in DevSim::pm once per solve.  Stage Q
+//     evaluated the equation of state, with an IEEE division and the branch over its kinds, at 1.69
+//     points per site in each sweep; now it reads two words.  The factor holds the (2/3)^2 of the two
+//     derivatives and the -1/12 of S5, so the stencils are d1s and j~ is the sum of stage J as it stands.
+//   - Stage Q is in packed FP32x2, a pair of x-neighbouring points per thread.
+//   - rho - rho0 leaves the ring (the own site's is loaded), which pays for a second q plane: one
+//     barrier per phase instead of two, at three CTAs per SM as before (75 KB each).
+//   - Two tensor copies per plane (all components of a field in one box) instead of four, and the
+//     z-derivative sums roll through their own updates instead of being copied from plane to plane.
+// Measured: 395 -> 317 us at 256^3, 119 -> 93 at 160^3, 66 -> 64 at 128^3 (one wave); the force kernel 231 -> 250 us at 256^3,
+// once per step.  72 bytes per site, 0.57 of the measured copy bandwidth at 256^3; bound by shared memory
+// (3.5 wavefronts per site) and the latency between its barriers.  Tried on the way: two sites per thread on 32 x 16 tiles
+// (16 warps per SM) 366 us, 512 threads on 32 x 16 tiles 397 us, packed stage Q alone 387 us.
+template <bool TMA>
+__device__ __forceinline__ void b_sweep_pm(const DevSim& p, int pair, const Blk bid)
+{
+    using SP = SweepPmPlan;
+    constexpr int TX = SP::TX, NT = SP::NT, UX = SP::UX, UP = SP::UP, QX = SP::QX, QP = SP::QP, PP = SP::PP, R = SP::R;
+    constexpr int HZ = 4;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) unsigned long long ring_bar[R];  // one per ring slot (TMA)
+    unsigned char* sm = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    float* su = reinterpret_cast<float*>(sm);              // [R][3][UP]: u
+    float* sp = reinterpret_cast<float*>(sm + SP::OFF_P);  // [2][2][PP]: the pressure pair, plane z in z & 1
+    float* sq = reinterpret_cast<float*>(sm + SP::OFF_Q);  // [2][6][QP]: q_ab, plane z in z & 1
+    const int tid = threadIdx.x;
+    const int x0 = bid.x * TX, y0 = bid.y * SP::TY;
+    const int z0 = bid.z * p.zb[TK_SWEEP], z1 = min(z0 + p.zb[TK_SWEEP], p.nz);
+    const int NPL = p.nx * p.ny;
+    const float* drho = cp<float>(p.rho);
+    const int cur = p.us[pair].cur;
+    const float* uold = cp<float>(p.uit[pair][cur]);
+    float* unew = mp<float>(p.uit[pair][cur ^ 1]);
+    const float c1 = float(p.us[pair].c1), c2 = float(p.us[pair].c2);  // this sweep's update (see k_us_ctl)
+    float* dvec = mp<float>(p.dvec[pair]);
+    const bool use_d = c1 != 0.f, keep_d = p.cheb != 0, use_j = p.rtol != 0.0;
+    // the thread's own site (stage J)
+    const int ix = tid % TX, iy = tid / TX;
+    const int gx = x0 + ix, gy = y0 + iy;
+    const bool own = gx < p.nx && gy < p.ny;
+    const int own_xy = gy * p.nx + gx;
+    float dmax = 0.f, jmax = 0.f;
+    // Plane copies by the threads: groups of G box columns, G the largest of 4, 2, 1 that divides nx (the boxes
+    // start at x0 - 4, so each group is G consecutive aligned sites, also across the periodic wrap).
+    const int G = !p.aligned16 ? 1 : p.nx % 4 == 0 ? 4 : p.nx % 2 == 0 ? 2 : 1;
+    constexpr int MG = (UP + NT - 1) / NT;
+    int goff[MG];  // in-plane lattice offset of the thread's groups; the pressure box is rows 2 .. 13 of u's
+#pragma unroll
+    for (int m = 0; m < MG; ++m) {
+        const int k = (tid + m * NT) * G;
+        goff[m] = k < UP ? wrapm(x0 - 4 + k % UX, p.nx) + p.nx * wrapm(y0 - 4 + k / UX, p.ny) : 0;
+    }
+    auto copy_plane = [&](auto gc, int zl, int sl) {
+        constexpr int GC = decltype(gc)::value;
+        const float* ub = uold + (long long)wrapc(zl, p.nz) * NPL;
+        const int zp = zl - 2;  // the pressure plane that goes with u's plane zl
+        const bool pr = zp >= z0 - 2 && zp < z1 + 2;
+        const float* pb = p.pm + (long long)wrapc(zp, p.nz) * NPL;
+        float* du = su + sl * 3 * UP;
+        float* dp = sp + (zp & 1) * 2 * PP;
+#pragma unroll
+        for (int m = 0; m < (UP / GC + NT - 1) / NT; ++m) {
+            const int k = (tid + m * NT) * GC;
+            if (k < UP) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) cp_async<GC * 4>(du + a * UP + k, ub + a * p.N + goff[m]);
+                if (pr && k >= 2 * UX && k < 2 * UX + PP) {
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) cp_async<GC * 4>(dp + a * PP + k - 2 * UX, pb + a * p.N + goff[m]);
+                }
+            }
+        }
+    };
+    auto fetch = [&](int zl, int sl) {
+        if (G == 4) copy_plane(std::integral_constant<int, 4>{}, zl, sl);
+        else if (G == 2) copy_plane(std::integral_constant<int, 2>{}, zl, sl);
+        else copy_plane(std::integral_constant<int, 1>{}, zl, sl);
+    };
+    // Tensor copies for tiles whose halo box stays inside the lattice in x and y (CTA-uniform).
+    bool tma = false;
+    if constexpr (TMA) {
+        tma = p.tma != 0 && x0 >= 4 && x0 + TX + 4 <= p.nx && y0 >= 4 && y0 + SP::TY + 4 <= p.ny;
+        if (tma) {
+            if (tid == 0) {
+#pragma unroll
+                for (int k = 0; k < R; ++k) mbar_init(&ring_bar[k], 1);
+                fence_mbar_init();
+                p.us[pair].tma = 1;  // reported by lbm_stats_get
+            }
+            __syncthreads();
+        }
+    }
+    unsigned phase = 0;        // parity of each ring slot's barrier phase that the next wait expects
+    int aborted_at = INT_MIN;  // plane whose tensor copies timed out
+    auto fetch_tma = [&](int zl, int sl) {
+        if (tid == 0) {
+            const int zp = zl - 2;
+            const bool pr = zp >= z0 - 2 && zp < z1 + 2;
+            unsigned long long* bar = &ring_bar[sl];
+            fence_proxy_async_smem();
+            mbar_expect_tx(bar, unsigned((3 * UP + (pr ? 2 * PP : 0)) * sizeof(float)));
+            tma_load_4d(su + sl * 3 * UP, &p.tmaps->u[pair][cur], bar, x0 - 4, y0 - 4, wrapc(zl, p.nz), 0);
+            if (pr) tma_load_4d(sp + (zp & 1) * 2 * PP, &p.tmaps->rho, bar, x0 - 4, y0 - 2, wrapc(zp, p.nz), 0);
+        }
+    };
+    // stage J inputs of the own site (j0', previous update, rho - rho0), fetched one plane ahead
+    float pj[3] = {0.f, 0.f, 0.f}, pd[3] = {0.f, 0.f, 0.f}, jr = 0.f;
+    auto fetch_j = [&](int zj) {
+        if (own && zj >= z0 && zj < z1) {
+            const int g = zj * NPL + own_xy;
+            jr = drho[g];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                pj[a] = plane<float>(p.j0pp, a)[g];
+                if (use_d) pd[a] = (dvec + a * p.N)[g];
+            }
+        }
+    };
+    // A[k][a]: sum over b of d_b q_ab at plane zs - 1 + k of the own site, as far as known before stage J
+    // of plane zs
+    float A[4][3];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) A[k][a] = 0.f;
+    float ju[3] = {0.f, 0.f, 0.f};  // own u of the plane that the next stage J finishes
+    // stage Q's pair of this thread: consecutive pairs of the row pitch, 18 of 20 in use
+    static_assert(UX / 2 * SP::QY <= NT, "one round of stage Q");
+    const bool q_on = tid < UX / 2 * SP::QY && tid % (UX / 2) < QX / 2;
+    const int qrow = tid / (UX / 2), qcol = 2 * (tid % (UX / 2));
+    int sl = (z0 - HZ + 8 * R) % R;  // ring slot of plane zl (z0 - HZ >= -4)
+    auto back = [&](int k) { return sl >= k ? sl - k : sl - k + R; };  // slot of plane zl - k
+    if (tma) fetch_tma(z0 - HZ, sl);
+    else fetch(z0 - HZ, sl);
+    cp_async_commit();
+    fetch_j(z0);
+    // Phase zl: stage J of plane zs = zl - 3, whose q the previous phase wrote, which finishes plane zs - 2, and
+    // stage Q of plane zq = zl - 2 into the other q plane; the last phase only finishes.
+    for (int zl = z0 - HZ; zl < z1 + HZ + 1; ++zl) {
+        bool late = false;
+        if (tma && zl < z1 + HZ) {  // plane zl's tensor copies have landed (the last phase loads none)
+            late = !mbar_wait(&ring_bar[sl], (phase >> sl) & 1u);
+            if (!late) phase ^= 1u << sl;
+        } else {
+            cp_async_wait<0>();  // plane zl has landed (this thread's copies)
+        }
+        // ... and everyone's copies; the previous phase is done
+        if (!tma) {
+            __syncthreads();
+        } else if (__syncthreads_or(late)) {
+            aborted_at = zl;
+            break;
+        }
+        const int sn = sl + 1 == R ? 0 : sl + 1;  // held plane zl - 5, read last in the previous phase
+        if (zl + 1 < z1 + HZ) {
+            if (tma) fetch_tma(zl + 1, sn);
+            else fetch(zl + 1, sn);
+        }
+        cp_async_commit();
+        const int zq = zl - 2, zs = zq - 1;
+        if (zs >= z0 - 2 && zs < z1 + 2) {  // stage J: plane zs
+            const float* qb = sq + (zs & 1) * SP::NQ * QP + (iy + 2) * QX + ix + 2;
+            float in[3] = {0.f, 0.f, 0.f};
+            if (zs >= z0 && zs < z1) {  // in-plane derivatives d_x q_ax + d_y q_ay
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const float* qx = qb + sym2<3>(a, 0) * QP;
+                    const float* qy = qb + sym2<3>(a, 1) * QP;
+                    in[a] = d1s(qx[-2], qx[-1], qx[1], qx[2]) + d1s(qy[-2 * QX], qy[-QX], qy[QX], qy[2 * QX]);
+                }
+            }
+            float done[3];  // plane zs - 2, complete: j~new (S5)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                // the share of q_az(zs) in the z derivatives of the planes zs - 2 .. zs + 2
+                const float v = qb[sym2<3>(a, 2) * QP];
+                done[a] = __fmaf_rn(-0.125f, v, A[0][a]);
+                A[0][a] = A[1][a] + v;
+                A[1][a] = A[2][a] + in[a];
+                A[2][a] = A[3][a] - v;
+                A[3][a] = 0.125f * v;
+            }
+            const int zc = zs - 2;
+            if (own && zc >= z0 && zc < z1) {
+                const int g = zc * NPL + own_xy;
+                const float rho = p.pf.rho0 + jr;
+                const float irho = 1.f / rho;
+                float m = 0.f;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const float res = __fmaf_rn(pj[a] + done[a], irho, -ju[a]);
+                    float d = c2 * res;
+                    if (use_d) d = __fmaf_rn(c1, pd[a], d);
+                    if (keep_d) (dvec + a * p.N)[g] = d;
+                    (unew + a * p.N)[g] = __fadd_rn(ju[a], d);
+                    m = max_nan(m, max_nan(fabsf(res), fabsf(d)));  // S6: see b_sweep
+                    if (use_j) jmax = fmaxf(jmax, fabsf(done[a]));
+                }
+                dmax = max_nan(dmax, rho * m);
+            }
+            fetch_j(zc + 1);
+        }
+        const int zj = zl - HZ;
+        if (zj >= z0 && zj < z1) {
+            const float* uc = su + back(4) * 3 * UP + (iy + 4) * UX + ix + 4;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) ju[a] = uc[a * UP];
+        }
+        if (q_on && zq >= z0 - 2 && zq < z1 + 2) {  // stage Q: plane zq
+            const int ui = (qrow + 2) * UX + qcol + 2;
+            const float* pl[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) pl[k] = su + back(4 - k) * 3 * UP + ui;
+            float2 du[3][3];  // [a][b] = 3/2 d_a u_b of the two points
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const float* c = pl[2] + b * UP;
+                du[0][b] = d1sx2(ld2<float>(c - 2), ld2<float>(c), ld2<float>(c + 2));
+                du[1][b] = d1s2(ld2<float>(c - 2 * UX), ld2<float>(c - UX), ld2<float>(c + UX), ld2<float>(c + 2 * UX));
+                du[2][b] = d1s2(ld2<float>(pl[0] + b * UP), ld2<float>(pl[1] + b * UP), ld2<float>(pl[3] + b * UP),
+                                ld2<float>(pl[4] + b * UP));
+            }
+            const float* pq = sp + (zq & 1) * 2 * PP + qrow * UX + qcol + 2;
+            const float2 P2 = ld2<float>(pq), PM2 = ld2<float>(pq + PP);
+            const float2 pdv = mul2(PM2, add2(add2(du[0][0], du[1][1]), du[2][2]));
+            float* qo = sq + (zq & 1) * SP::NQ * QP + qrow * QX + qcol;
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = a; b < 3; ++b) {
+                    const float2 sd = add2(du[b][a], du[a][b]);
+                    *reinterpret_cast<float2*>(qo + sym2<3>(a, b) * QP) = a == b ? fma2(P2, sd, pdv) : mul2(P2, sd);
+                }
+        }
+        sl = sn;
+    }
+    cp_async_wait<0>();
+    if (aborted_at != INT_MIN) {
+        // the plane in flight (at the abort, plane aborted_at) has landed or timed out before the CTA ends
+        if (tid == 0) {
+            atomicOr(p.status, STB_TIMEOUT);
+            (void)mbar_wait(&ring_bar[sl], (phase >> sl) & 1u);
+        }
+        dmax = __int_as_float(0x7f800000);  // the residual reads as infinite: the control kernel ends the solve
+    }
+    // NaN -> +inf, which orders above every finite residual
+    const double dmax_d = dmax == dmax ? double(dmax) : __longlong_as_double(0x7ff0000000000000ll);
+    block_max2(dmax_d, double(jmax), &p.us[pair].resid_bits, &p.us[pair].jmax_bits);
+}
+template <bool TMA>
+__global__ void __launch_bounds__(SweepPmPlan::NT, 3) k_sweep_pm(DevSim p, int pair, int mode)
+{
+    if (mode != SWEEP_ALONE && !p.us[pair].running) return;  // launched ahead, and the solve has stopped
+    b_sweep_pm<TMA>(p, pair, launch_blk());
+}
+
 // Equation of state of two sites (see eos_full, cs2_delta).  Every operation is written out, and the psi-sine
 // form is one function that is not inlined, so that a site's result does not depend on which of the
 // two words it has: left to the compiler, the two scalar copies contracted differently in rare cases.
@@ -1780,6 +2068,14 @@ __device__ __forceinline__ void b_force(const DevSim& p, int pair, const Blk bid
                 plane<T>(p.fpp, a)[g] = fa;
                 plane<T>(p.j0pp, a)[g] = j;
                 u0[a * p.N + g] = (U(j) + pw[a]) / rho;
+            }
+            if constexpr (D == 3 && sizeof(T) == 4 && sizeof(U) == 4) {
+                if (p.pm) {  // the pressure pair of b_sweep_pm
+                    T P, DP, PM, RPP;
+                    eos_full<T>(p, rs, P, DP, PM, RPP);
+                    p.pm[g] = T(-1.0 / 27.0) * P;
+                    p.pm[p.N + g] = T(-1.0 / 27.0) * PM;
+                }
             }
         }
         if (zc >= z0 && zc < z1) fetch_own(zc + 1);
@@ -2827,6 +3123,17 @@ __global__ void __launch_bounds__(Tile<Lat<LAT>::D>::THREADS, sizeof(U) == 4 ? 2
     }
 }
 
+static __global__ void __launch_bounds__(SweepPmPlan::NT, 3) kb_sweep_pm(const DevSim* sims, const BatchWork* w, int pair)
+{
+    const int n = w->nslot, total = w->tstart[TK_SWEEP][n];
+    for (int item = blockIdx.x; item < total; item += gridDim.x) {
+        const int k = batch_slot(w->tstart[TK_SWEEP], n, item);
+        if (!w->live[k] || !sims[k].us[pair].running) continue;
+        b_sweep_pm<false>(sims[k], pair, batch_tile(w, TK_SWEEP, k, item - w->tstart[TK_SWEEP][k]));
+        __syncthreads();
+    }
+}
+
 // One warp: the control step of every slot whose solve is running; the loop goes on while any is.
 static __global__ void kb_us_ctl(const DevSim* sims, const BatchWork* w, int pair, cudaGraphConditionalHandle h)
 {
@@ -3223,6 +3530,16 @@ KernelTable make_table(bool read_pops)
     cudaFuncSetAttribute(t.derivs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_derivs));
     cudaFuncSetAttribute(t.collide, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_collide));
     if constexpr (kPairCollide<LAT, T, S, U>) {
+        t.sweep = (const void*)k_sweep_pm<false>;
+        t.sweep_tma = (const void*)k_sweep_pm<true>;
+        t.kb_sweep = (const void*)kb_sweep_pm;
+        t.tile[TK_SWEEP] = TileShape{SweepPmPlan::TX, SweepPmPlan::TY, SweepPmPlan::NT};
+        t.smem_sweep = SweepPmPlan::BYTES;
+        t.sweep_box[0] = SweepPmPlan::UX;
+        t.sweep_box[1] = SweepPmPlan::UY;
+        t.pm_rows = SweepPmPlan::QY;
+        for (const void* f : {t.sweep, t.sweep_tma, t.kb_sweep})
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t.smem_sweep));
         t.pair_collide[0] = pair_collide<S, 32>(read_pops);
         t.pair_collide[1] = pair_collide<S, 64>(read_pops);
         t.pair_derivs = (const void*)k_derivs_pair;
