@@ -3223,6 +3223,18 @@ __global__ void k_init_eq(DevSim p, const double* rho_in, const double* u_in, in
     T u[3] = {T(0), T(0), T(0)};
     if (u_in)
 #pragma unroll
+// float to double on integer units, to the bit what the conversion instruction gives: that runs on the FP64 units,
+// at 1/64 of the FP32 rate, and with the FP64 addition of the export convention made the export of 59
+// populations FP64-bound (96^3 FP32 deviations 229 -> 151 us; its bytes take 94).  Zeros and normal values here;
+// subnormal, infinite and NaN ones through the instruction.  (The 16-bit and local-reference exports
+// were no faster with it, nor was the import with an integer rounding to float: they convert as before.)
+__device__ __forceinline__ double to_double(float v)
+{
+    const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u) return __hiloint2double(int((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), int(b << 29));
+    if (a == 0) return __hiloint2double(int(b), 0);
+    return double(v);
+}
         for (int a = 0; a < L::D; ++a) u[a] = T(u_in[a * p.N + s]);
     const T drs = T(rho_in[s] - p.rho0);
     T cs2, dcs2;
@@ -3308,7 +3320,14 @@ __device__ __forceinline__ double pop_full(const DevSim& p, int b, int i, long l
 {
     using L = Lat<LAT>;
     using C = Codec<S>;
-    const double v = pop_raw<LAT, S, double>(p, b, i, s);
+    if constexpr (!C::EXACT) return pop_raw<LAT, S, double>(p, b, i, s);
+    if (i == 0) {  // the exact pair
+        const float2 r = cp<float2>(p.pop0[b])[s];
+        const double v = double(r.x) + double(r.y);
+        if (C::LOC) return v + double(p.wref[b][s]);
+        return v + (C::DEV ? p.off[0] : 0.0);
+    }
+    const float v = pop_raw<LAT, S, float>(p, b, i, s);
     if (C::LOC) {
         // the decoded value every density sum uses: fl(stored + sender's reference) for the
         // moving populations, the exact pair plus the own reference for the rest population
@@ -3316,7 +3335,8 @@ __device__ __forceinline__ double pop_full(const DevSim& p, int b, int i, long l
         const int x = int(s % p.nx), y = int((s / p.nx) % p.ny), z = int(s / ((long long)p.nx * p.ny));
         return double(__fadd_rn(float(v), p.wref[b][L::shell(i) * p.N + sender<LAT>(p, x, y, z, i)]));
     }
-    return v + (C::DEV ? p.off[L::shell(i)] : 0.0);
+    const double d = sizeof(typename C::type) == 4 ? to_double(v) : double(v);
+    return C::DEV ? d + p.off[L::shell(i)] : d;
 }
 
 template <int LAT, typename T, typename U>
@@ -3327,10 +3347,14 @@ __global__ void k_fields_out(DevSim p, int pair, double* rho_out, double* u_out)
     if (s >= p.N) return;
     const T rs = phys<T>(p).rho0 + cp<T>(p.rho)[s];
     const U* uu = cp<U>(p.uit[pair][p.us[pair].cur]);
-    if (rho_out) rho_out[s] = double(rs);
+    auto wide = [](auto v) {
+        if constexpr (sizeof(v) == 4) return to_double(v);
+        else return double(v);
+    };
+    if (rho_out) rho_out[s] = wide(rs);
     if (u_out)
 #pragma unroll
-        for (int a = 0; a < L::D; ++a) u_out[a * p.N + s] = double(uu[a * p.N + s]);
+        for (int a = 0; a < L::D; ++a) u_out[a * p.N + s] = wide(uu[a * p.N + s]);
 }
 
 template <int LAT, int S>
