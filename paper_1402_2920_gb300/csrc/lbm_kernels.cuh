@@ -3203,6 +3203,18 @@ static __global__ void k_reset(DevSim p)
 // ---------------------------------------------------------------------------
 // Initial condition, field and population transfer, conservation sums
 // ---------------------------------------------------------------------------
+// float to double on integer units, to the bit what the conversion instruction gives: that runs on the FP64 units,
+// at 1/64 of the FP32 rate, and with the FP64 addition of the export convention made the export of 59
+// populations FP64-bound (96^3 FP32 deviations 229 -> 151 us; its bytes take 94).  Zeros and normal values here;
+// subnormal, infinite and NaN ones through the instruction.  (The 16-bit and local-reference exports
+// were no faster with it, nor was the import with an integer rounding to float: they convert as before.)
+__device__ __forceinline__ double to_double(float v)
+{
+    const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u) return __hiloint2double(int((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), int(b << 29));
+    if (a == 0) return __hiloint2double(int(b), 0);
+    return double(v);
+}
 // w_k(c_s^2(rho)) in FP64 (initialisation only)
 template <int LAT>
 __device__ __forceinline__ double lat_weight_d(int k, const DevSim& p, double rho)
@@ -3223,18 +3235,6 @@ __global__ void k_init_eq(DevSim p, const double* rho_in, const double* u_in, in
     T u[3] = {T(0), T(0), T(0)};
     if (u_in)
 #pragma unroll
-// float to double on integer units, to the bit what the conversion instruction gives: that runs on the FP64 units,
-// at 1/64 of the FP32 rate, and with the FP64 addition of the export convention made the export of 59
-// populations FP64-bound (96^3 FP32 deviations 229 -> 151 us; its bytes take 94).  Zeros and normal values here;
-// subnormal, infinite and NaN ones through the instruction.  (The 16-bit and local-reference exports
-// were no faster with it, nor was the import with an integer rounding to float: they convert as before.)
-__device__ __forceinline__ double to_double(float v)
-{
-    const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
-    if (a - 0x00800000u < 0x7f000000u) return __hiloint2double(int((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), int(b << 29));
-    if (a == 0) return __hiloint2double(int(b), 0);
-    return double(v);
-}
         for (int a = 0; a < L::D; ++a) u[a] = T(u_in[a * p.N + s]);
     const T drs = T(rho_in[s] - p.rho0);
     T cs2, dcs2;
@@ -3331,9 +3331,8 @@ __device__ __forceinline__ double pop_full(const DevSim& p, int b, int i, long l
     if (C::LOC) {
         // the decoded value every density sum uses: fl(stored + sender's reference) for the
         // moving populations, the exact pair plus the own reference for the rest population
-        if (i == 0) return v + double(p.wref[b][s]);
         const int x = int(s % p.nx), y = int((s / p.nx) % p.ny), z = int(s / ((long long)p.nx * p.ny));
-        return double(__fadd_rn(float(v), p.wref[b][L::shell(i) * p.N + sender<LAT>(p, x, y, z, i)]));
+        return double(__fadd_rn(v, p.wref[b][L::shell(i) * p.N + sender<LAT>(p, x, y, z, i)]));
     }
     const double d = sizeof(typename C::type) == 4 ? to_double(v) : double(v);
     return C::DEV ? d + p.off[L::shell(i)] : d;
