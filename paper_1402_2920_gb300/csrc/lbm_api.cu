@@ -457,8 +457,8 @@ void setup_sweep_maps(lbm_sim* s)
     bool ok = true;
     for (int pr = 0; pr < 2; ++pr)
         for (int b = 0; b < 2; ++b)
-            ok = ok && encode_plane_map(&m.u[pr][b], dv.uit[pr][b], 3, s->kt.usize, dv, bx, by, dv.pm ? 3 : 1);
-    ok = ok && (dv.pm ? encode_plane_map(&m.rho, dv.pm, 2, sizeof(float), dv, bx, s->kt.pm_rows, 2)
+            ok = ok && encode_plane_map(&m.u[pr][b], dv.uit[pr][b], 3, s->kt.usize, dv, bx, by, dv.pm_scaled ? 3 : 1);
+    ok = ok && (dv.pm_scaled ? encode_plane_map(&m.rho, dv.pm, 2, sizeof(float), dv, bx, s->kt.pm_rows, 2)
                       : encode_plane_map(&m.rho, dv.rho, 1, s->kt.tsize, dv, bx, by, 1));
     void* dm = nullptr;
     ok = ok && dev_alloc(s, &dm, sizeof(SweepMaps)) == LBM_OK;
@@ -820,11 +820,6 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
     if (s->kt.exact) rc = rc ? rc : dev_alloc(s, &dv.rho_lo, N * sizeof(float));
     rc = rc ? rc : dev_alloc(s, &dv.rho, N * T);
     rc = rc ? rc : dev_alloc(s, &dv.j0p, 3 * N * T);
-    if (s->kt.pm_rows) {
-        void* w = nullptr;
-        rc = rc ? rc : dev_alloc(s, &w, 2 * N * sizeof(float));
-        dv.pm = static_cast<float*>(w);
-    }
     rc = rc ? rc : dev_alloc(s, &dv.f, 3 * N * T);
     for (int pr = 0; pr < 2; ++pr)
         for (int b = 0; b < 2; ++b) rc = rc ? rc : dev_alloc(s, &dv.uit[pr][b], 3 * N * U);
@@ -842,6 +837,8 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
         rc = rc ? rc : dev_alloc(s, &dv.dvec[1], 3 * N * U);
     }
     rc = rc ? rc : dev_alloc(s, &dv.aux, size_t(MAX_AUX) * N * T);
+    dv.pm = dv.aux;
+    dv.pm_scaled = s->kt.pm_rows ? 1 : 0;
     if (!rc) {
         for (int c = 0; c < MAX_AUX; ++c) dv.auxp[c] = static_cast<char*>(dv.aux) + size_t(c) * N * T;
         for (int a = 0; a < 3; ++a) {

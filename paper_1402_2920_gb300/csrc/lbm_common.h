@@ -127,8 +127,9 @@ struct DevSim {
     void* jt_warm;        // U [nw][3][N]: j~ = rho u - j0' of the last step, the warm start (Sec. IX),
                           // and with the extrapolated start (warm = 2) that of the step before
     void* aux;            // T [26][N]: A, B_ab, C_a, the local part of Sigma_ab, Xi'_abc
-    float* pm;            // [2][N]: -p/27 and -(p - rho p')/27 of every site, left by the force kernel for b_sweep_pm
-                          // (3D FP32 deviations with FP32 sweeps; else null)
+    void* pm;             // U [2][N]: p and p - rho p' of every site, left by the force kernel for FP64 sweeps and
+                          // b_sweep_pm in the first planes of aux, which is free until the derivatives
+    int pm_scaled;        // 1: both times -1/27 (b_sweep_pm)
     float* wref[2];       // [NSHELL][N] per population buffer (local-reference storages): w_k(c_s^2(rho)) rho
                           // of every site at the collision that sent the populations in that buffer
     UsolveState* us;      // [2]: pair 0 and pair 1

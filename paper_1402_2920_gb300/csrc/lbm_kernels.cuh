@@ -1365,6 +1365,21 @@ __device__ __forceinline__ void b_sweep(const DevSim& p, int pair, const Blk bid
         cp_async_commit();
     }
     fetch_j(z0);
+    // Stage Q's pair of points of this thread.  FP64 sweeps read p and p - rho p' of the points, which the force
+    // kernel leaves once per solve, at the start of the phase: evaluated here at 1.69 points per site, with a
+    // division, they took 13 % of a kernel that is bound by the FP64 units (48^3 121 -> 105 us).  FP32
+    // sweeps evaluate them: loading was no faster (128^3 65.7 against 67.6 us).
+    constexpr bool LOAD_P = sizeof(U) == 8;
+    constexpr int PX = UX / 2;  // point pairs per row of the pitch
+    static_assert(QY * PX <= NT, "one round of stage Q");
+    const int qx = 2 * (tid % PX), qy = tid / PX;
+    const bool q_on = tid < QY * PX && qx < QX;
+    const U* pm = cp<U>(p.pm);
+    int qoff[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        qoff[h] = LOAD_P && q_on ? wrapm(x0 - 2 + qx + h, p.nx) + p.nx * wrapm(y0 - 2 + qy, p.ny) : 0;
+    U qP[2] = {U(0), U(0)}, qPM[2] = {U(0), U(0)};
     // q_ab of plane z lives in the q plane buffer (or one of two, with NQB = 2)
     auto qbuf = [&](int z) { return sq + (SP::NQB == 2 ? (z & 1) : 0) * NQ * QP; };
     auto qplane = [&](int z) { return D == 2 ? z == 0 : (z >= z0 - 2 && z < z1 + 2); };
@@ -1404,6 +1419,14 @@ __device__ __forceinline__ void b_sweep(const DevSim& p, int pair, const Blk bid
             cp_async_commit();
         }
         const int zq = zl - HZ / 2, zs = zq - 1;
+        if (LOAD_P && q_on && qplane(zq)) {
+            const U* b = pm + (D == 3 ? (long long)wrapc(zq, p.nz) * NP : 0);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                qP[h] = b[qoff[h]];
+                qPM[h] = b[p.N + qoff[h]];
+            }
+        }
         if (qplane(zs)) {  // stage J: plane zs, whose q the previous phase wrote
             const U* qb = qbuf(zs);
             const int qi = (iy + 2) * UX + ix + 2;
@@ -1478,16 +1501,13 @@ __device__ __forceinline__ void b_sweep(const DevSim& p, int pair, const Blk bid
             jr = U(sr[slot(zj) * UP + ui]);
         }
         if (SP::NQB == 1 && D == 3) __syncthreads();  // stage J's reads of the q plane are done
-        if (qplane(zq)) {  // stage Q: plane zq, two x-neighbouring points per thread (64-bit reads)
+        if (q_on && qplane(zq)) {  // stage Q: plane zq, two x-neighbouring points per thread (64-bit reads)
             U* qb = qbuf(zq);
             const U* pl[5];
 #pragma unroll
             for (int k = 0; k < 5; ++k) pl[k] = su + slot(D == 3 ? zq - 2 + k : 0) * D * UP;
             const T* rq = sr + slot(zq) * UP;
-            constexpr int PX = UX / 2;  // point pairs per row of the pitch
-            for (int t = tid; t < QY * PX; t += NT) {
-                const int qx = 2 * (t % PX), qy = t / PX;
-                if (qx >= QX) continue;
+            {
                 const int k = qy * UX + qx;      // even: the pair is 2-element aligned
                 const int ui = k + 2 * UX + 2;   // (qy + 2) UX + qx + 2
                 U du[2][3][3];                   // [point][a][b] = d_a u_b
@@ -1511,8 +1531,8 @@ __device__ __forceinline__ void b_sweep(const DevSim& p, int pair, const Blk bid
                 U qv[2][NQ];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    U P, DP, PM, RPP;
-                    eos_full<U>(p, phys<U>(p).rho0 + U(rq[ui + h]), P, DP, PM, RPP);
+                    U P = qP[h], PM = qPM[h], DP, RPP;
+                    if (!LOAD_P) eos_full<U>(p, phys<U>(p).rho0 + U(rq[ui + h]), P, DP, PM, RPP);
                     U div = U(0);
 #pragma unroll
                     for (int a = 0; a < D; ++a) div += du[h][a][a];
@@ -1621,7 +1641,8 @@ struct SweepPmPlan {
 };
 
 // S3-S6 fused for the 3D FP32-deviation storage: b_sweep's march and stages (see there), leaner.
-//   - The force kernel leaves -p/27 and -(p - rho p')/27 of every site in DevSim::pm once per solve.  Stage Q
+//   - The force kernel leaves -p/27 and -(p - rho p')/27 of every site in DevSim::pm once per solve (planes of
+//     aux, which is free until the derivatives).  Stage Q
 //     evaluated the equation of state, with an IEEE division and the branch over its kinds, at 1.69
 //     points per site in each sweep; now it reads two words.  The factor holds the (2/3)^2 of the two
 //     derivatives and the -1/12 of S5, so the stencils are d1s and j~ is the sum of stage J as it stands.
@@ -1678,7 +1699,7 @@ __device__ __forceinline__ void b_sweep_pm(const DevSim& p, int pair, const Blk 
         const float* ub = uold + (long long)wrapc(zl, p.nz) * NPL;
         const int zp = zl - 2;  // the pressure plane that goes with u's plane zl
         const bool pr = zp >= z0 - 2 && zp < z1 + 2;
-        const float* pb = p.pm + (long long)wrapc(zp, p.nz) * NPL;
+        const float* pb = cp<float>(p.pm) + (long long)wrapc(zp, p.nz) * NPL;
         float* du = su + sl * 3 * UP;
         float* dp = sp + (zp & 1) * 2 * PP;
 #pragma unroll
@@ -2069,13 +2090,12 @@ __device__ __forceinline__ void b_force(const DevSim& p, int pair, const Blk bid
                 plane<T>(p.j0pp, a)[g] = j;
                 u0[a * p.N + g] = (U(j) + pw[a]) / rho;
             }
-            if constexpr (D == 3 && sizeof(T) == 4 && sizeof(U) == 4) {
-                if (p.pm) {  // the pressure pair of b_sweep_pm
-                    T P, DP, PM, RPP;
-                    eos_full<T>(p, rs, P, DP, PM, RPP);
-                    p.pm[g] = T(-1.0 / 27.0) * P;
-                    p.pm[p.N + g] = T(-1.0 / 27.0) * PM;
-                }
+            if (sizeof(U) == 8 || p.pm_scaled) {  // p and p - rho p' for the sweeps, scaled for b_sweep_pm (see there)
+                U P, DP, PM, RPP;
+                eos_full<U>(p, phys<U>(p).rho0 + U(R(0, 0, 0)), P, DP, PM, RPP);
+                U* pm = mp<U>(p.pm);
+                pm[g] = p.pm_scaled ? U(-1.0 / 27.0) * P : P;
+                pm[p.N + g] = p.pm_scaled ? U(-1.0 / 27.0) * PM : PM;
             }
         }
         if (zc >= z0 && zc < z1) fetch_own(zc + 1);
