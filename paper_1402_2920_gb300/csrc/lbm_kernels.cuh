@@ -14,6 +14,8 @@
 //                       parts of Sigma and the whole Xi'
 //   k_collide   S11,S12 nested derivatives (tiled), Sigma, per-velocity collision,
 //                       push streaming n_i(r + c_i) = n_i + Delta_i
+// For 3D FP32 deviations k_sweep_pm takes the place of k_sweep and, with nx even, k_derivs_pair and
+// k_collide_pair those of k_derivs and k_collide: packed FP32x2 arithmetic, two sites per instruction.
 #pragma once
 
 #include <climits>
@@ -1653,7 +1655,7 @@ struct SweepPmPlan {
 //     z-derivative sums roll through their own updates instead of being copied from plane to plane.
 // Measured: 395 -> 317 us at 256^3, 119 -> 93 at 160^3, 66 -> 64 at 128^3 (one wave); the force kernel 231 -> 250 us at 256^3,
 // once per step.  72 bytes per site, 0.57 of the measured copy bandwidth at 256^3; bound by shared memory
-// (3.5 wavefronts per site) and the latency between its barriers.  Tried on the way: two sites per thread on 32 x 16 tiles
+// (4.0 wavefronts per site) and the latency between its barriers.  Tried on the way: two sites per thread on 32 x 16 tiles
 // (16 warps per SM) 366 us, 512 threads on 32 x 16 tiles 397 us, packed stage Q alone 387 us.
 template <bool TMA>
 __device__ __forceinline__ void b_sweep_pm(const DevSim& p, int pair, const Blk bid)
