@@ -113,8 +113,10 @@ typedef struct {
                               the iteration (g as for usolve_omega; needs the density range),
                               about half the sweeps of the best plain relaxation on noise.
                               Solves of smooth flows open with plain sweeps, which are the
-                              faster there, and a solve whose residual grows, or stalls near
-                              the tolerance, ends with them.  The fixed point, and so the result up to the tolerance, is unchanged */
+                              faster there (never where usolve_max_iter is 10 or less), and a
+                              solve whose residual grows, or stalls near the tolerance, ends
+                              with them.  The fixed point, and so the result up to the
+                              tolerance, is unchanged                                        */
 } lbm_params;
 
 typedef struct {

@@ -9,36 +9,12 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "lbm_usolve.h"
+
 namespace lbm {
 
 enum Store { ST_F32 = 0, ST_F32_DEV = 1, ST_F16_DEV = 2, ST_BF16_DEV = 3, ST_F64 = 4, ST_F32_LOC = 5, ST_F16_LOC = 6,
              ST_BF16_LOC = 7 };
-
-// Device-resident state of one implicit u-solve (Sec. IX): which of the two
-// j~ buffers is current, the sweep counter and the residual reductions.
-struct UsolveState {
-    unsigned long long resid_bits;  // atomicMax over |j~new - j~| (non-negative double bits)
-    unsigned long long jmax_bits;   // atomicMax over |j~new|
-    int cur;                        // buffer holding the current j~
-    int iter;                       // sweeps of the solve in progress
-    int iters_last;                 // sweeps of the last finished solve
-    int iters_max;                  // largest sweep count since init
-    double resid_last;              // residual of the last sweep: after a solve, its final one
-    int converged;                  // 1 once the last solve met its tolerance
-    int running;                    // 1 from k_us_begin until the control kernel stops the loop
-    long long sweeps_total;         // sweeps since the last reset
-    // the update of the next sweep: d = c1 d_prev + c2 (J(j~) - j~), j~ += d
-    double c1, c2;
-    double cheb_rho;                // Chebyshev recurrence variable
-    double cheb_sigma, cheb_delta;  // this solve's spectrum [1 - g, 1] of I - A (theta = 1 - g/2)
-    double gain;                    // this solve's bound g, from the density range of the state
-    double resid_min;               // smallest residual of the solve so far (divergence guard)
-    int mode;                       // 1: Chebyshev sweeps, 2: plain sweeps of a Chebyshev solve, 0: plain
-                                    // relaxation
-    int wsel;                       // pair 0: the warm-start buffer holding the newest j~ (see jwp)
-    int tma;                        // 1 once a sweep of this solve loaded planes by tensor copies
-    int opened;                     // 1: this solve (after it: the last one) opened with plain sweeps
-};
 
 // What the host reads back of a simulation: one device block, one copy.
 struct HostView {
@@ -51,19 +27,6 @@ struct HostView {
 // kernels prefetch into L2 (measured at 256^3)
 constexpr int kCollideLead = 1;
 constexpr int kDerivsLead = 1;
-
-// Plain sweeps inside Chebyshev-accelerated solves (32- and 64-bit storages).  J multiplies smooth
-// modes by almost zero, so on the smooth residual of a steady flow one plain sweep does what takes
-// Chebyshev five; on noise Chebyshev gains a factor 4 per sweep and plain 2.  A solve opens with plain
-// sweeps when the last one, opened by Chebyshev, took kPlainOpen to kPlainOpenMost sweeps, or opened
-// plainly and took fewer than kPlainOpen; it goes on plainly while that halves the residual, and
-// within kPlainNear tolerances.  A Chebyshev solve that no longer halves its residual within
-// kStallNear tolerances ends plainly: u of size 0.03 rounds at 2e-9 in FP32, and updates of 1.6
-// residuals met that rounding at the 5e-9 tolerance.  Longer solves (the noisy start of a quench)
-// stay Chebyshev from first to last: ended plainly, they took 4 % fewer sweeps but left twice the
-// error against FP64.
-constexpr int kPlainOpen = 4, kPlainOpenMost = 5;
-constexpr double kPlainNear = 8.0, kStallNear = 2.0;
 
 // The tiled kernels: each has its tile, its z-slab depth and so its grid.
 enum TiledKernel { TK_FORCE = 0, TK_SWEEP, TK_DERIVS, TK_COLLIDE, kTiled };
@@ -149,7 +112,7 @@ struct DevSim {
     double omega;                    // relaxation of the u-solve sweep (1 = the plain iteration);
                                      // 0: 2/(2 - g) with g the bound of each solve
     int cheb;                        // Chebyshev acceleration of the sweeps: 1 with plain sweeps where they
-                                     // are the faster (kPlainOpen), 2 throughout, 0 none
+                                     // are the faster (lbm_usolve.h), 2 throughout, 0 none
     double s2max;                    // max over k of |s(k)|^2 of the first-derivative symbol (1D)
     void* dvec[2];                   // U [3][N]: previous update of the u-solve, pair 0 and 1
     int maxit;

@@ -560,15 +560,6 @@ static __device__ double frozen_gain(const DevSim& p, double rho)
     return p.d * p.s2max / 12.0 * fmax(3.0 * cs2 - DP, cs2);
 }
 
-// First step of a Chebyshev semi-iteration from the current iterate: x += r / theta.
-static __device__ __forceinline__ void cheb_first(UsolveState& u)
-{
-    u.mode = 1;
-    u.cheb_rho = 1.0 / u.cheb_sigma;
-    u.c1 = 0.0;
-    u.c2 = 1.0 / (1.0 - u.cheb_delta);
-}
-
 // One warp (lane 0..31) per solve: the reductions are spread over the lanes (one thread took
 // 22 us per step, most of it in the 17 FP64 gain evaluations one after the other).
 static __device__ void b_us_begin(const DevSim& p, int pair, int lane)
@@ -597,34 +588,7 @@ static __device__ void b_us_begin(const DevSim& p, int pair, int lane)
     for (int o = 16; o > 0; o >>= 1) g = fmax(g, __shfl_xor_sync(0xffffffffu, g, o));
     if (lane != 0) return;
     g = fmin(0.95, 1.02 * g);
-    u.gain = g;
-    u.cheb_delta = 0.5 * g;
-    u.cheb_sigma = (1.0 - 0.5 * g) / (0.5 * g);
-    u.iter = 0;
-    u.resid_bits = 0ull;
-    u.jmax_bits = 0ull;
-    u.converged = 0;
-    u.running = 1;
-    u.tma = 0;
-    u.resid_min = 1e300;
-    // Whether this solve opens with plain sweeps (see kPlainOpen in lbm_common.h), from the run's last
-    // solve, which pair 1 reads too: what lbm_fields does depends on the run's state alone.
-    const UsolveState& run = p.us[0];
-    const bool plain = p.cheb == 1 && (run.opened ? run.iters_last < kPlainOpen
-                                                  : run.iters_last >= kPlainOpen && run.iters_last <= kPlainOpenMost);
-    u.opened = plain ? 1 : 0;
-    u.resid_last = 1e300;
-    if (plain) {
-        u.mode = 2;
-        u.c1 = 0.0;
-        u.c2 = 1.0;
-    } else if (p.cheb) {
-        cheb_first(u);
-    } else {       // plain relaxation x += omega r (omega = 0: 2/(2 - g))
-        u.mode = 0;
-        u.c1 = 0.0;
-        u.c2 = p.omega > 0.0 ? p.omega : 2.0 / (2.0 - g);
-    }
+    usolve_open(u, p.us[0], p.cheb, p.omega, p.maxit, g);
 }
 static __global__ void k_us_begin(DevSim p, int pair) { b_us_begin(p, pair, threadIdx.x & 31); }  // one warp
 
@@ -645,33 +609,7 @@ static __device__ bool b_us_ctl(const DevSim& p, int pair)
     else if (stop && !conv) atomicOr(p.status, STB_USOLVE_CAP);
     u.resid_bits = 0ull;
     u.jmax_bits = 0ull;
-    // Coefficients of the next sweep: Chebyshev semi-iteration for the real spectrum [1 - g, 1] of
-    // I - A, or plain sweeps, whose update is the residual itself.  resid_last holds the residual
-    // of the sweep before.  A residual four times above the best one so far means the spectral bound
-    // was too small: plain sweeps from there on (mode 0).
-    if (p.cheb) {
-        const double lim = p.tol + p.rtol * jm;
-        const bool halved = r <= 0.5 * u.resid_last;
-        if (u.mode == 1 && !bad && r > 4.0 * u.resid_min) u.mode = 0;
-        bool plain = u.mode == 0;
-        if (u.opened)  // plain as long as it pays, and near the tolerance
-            plain = plain || u.iter == 1 || r <= kPlainNear * lim || (u.mode == 2 && halved);
-        else if (p.cheb == 1)  // a Chebyshev update is 1.6 residuals: near the tolerance it can stall on
-                               // the rounding of u where a plain one would end
-            plain = plain || u.mode == 2 || (r <= kStallNear * lim && !halved);
-        if (plain) {
-            u.mode = u.mode == 0 ? 0 : 2;
-            u.c1 = 0.0;
-            u.c2 = 1.0;
-        } else if (u.mode == 2) {
-            cheb_first(u);
-        } else {
-            const double rn = 1.0 / (2.0 * u.cheb_sigma - u.cheb_rho);
-            u.c1 = rn * u.cheb_rho;
-            u.c2 = 2.0 * rn / u.cheb_delta;
-            u.cheb_rho = rn;
-        }
-    }
+    if (p.cheb && !bad) usolve_next(u, p.cheb, r, p.tol + p.rtol * jm);
     u.resid_last = r;
     u.resid_min = r < u.resid_min ? r : u.resid_min;
     if (stop) {
