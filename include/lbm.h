@@ -185,8 +185,8 @@ int lbm_set_populations(lbm_sim* sim, const double* in, int on_device);
  * (may be NULL) and returns Q (21 or 59), or LBM_E_INVALID_ARG. */
 int lbm_velocities(int lattice, int* c_out);
 
-/* Conservation sums (FP64, fixed reduction order), step counter and u-solve
- * statistics.  Synchronises. */
+/* Conservation sums (FP64 or more exactly, fixed reduction order), step counter and
+ * u-solve statistics.  Synchronises. */
 int lbm_stats_get(lbm_sim* sim, lbm_stats* out);
 
 /* Kernel timing (tracing aid).  Each kernel of the time step is launched reps >= 1

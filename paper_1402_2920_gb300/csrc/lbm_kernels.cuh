@@ -3349,14 +3349,34 @@ __global__ void k_pops_in(DevSim p, const double* in, int dst)
 constexpr int RED_BLOCK = kRedBlock;
 constexpr int RED_GRID = kRedGrid;
 
-// The reduced storages sum a site's populations as float pairs and add the site's four totals in FP64.
-// GB300 does one FP64 addition in 64 FP32 ones: with every population converted and added in FP64 the sums
-// of a 256^3 D3Q59 state took 12.4 ms, of a 128^3 one 1.6 ms, against 0.64 and 0.08 ms for reading it.  The
-// density adds the stored floats with error-free sums (acc2), the momentum the differences of
-// opposite populations, each an exact pair; both keep 2^-48 of the deviations, where FP64 sums of n_i
-// themselves keep 2^-53 of n_i.
+// GB300 does one FP64 addition in 64 FP32 ones: with every population converted and added in FP64 lbm_stats_get took
+// 12.4 ms of a 256^3 D3Q59 state and 1.6 ms of a 128^3 one, against 0.64 and 0.08 ms for reading it.  So the storages
+// that hold floats are summed in three floats, with error-free additions in the low parts too: 2^-70 of the
+// sum where an FP64 sum keeps 2^-53, and the three become one double once per thread.  1.22 and 0.19 ms, bound by
+// FP32 additions (2,000 per site); pairs of floats took 0.82 and 0.14 ms, and kept 2^-48.
+struct Sum3 {
+    float h, m, l;
+    __device__ __forceinline__ void low(float v)  // v no larger than the roundings of h
+    {
+        float e;
+        two_sum(m, v, m, e);
+        l = __fadd_rn(l, e);
+    }
+    __device__ __forceinline__ void add(float v)
+    {
+        float e;
+        two_sum(h, v, h, e);
+        low(e);
+    }
+    // an overflow, an infinity or a NaN on the way leaves h or m one
+    __device__ __forceinline__ bool finite() const { return isfinite(h) && isfinite(m); }
+    __device__ __forceinline__ double value() const { return (double(h) + double(m)) + double(l); }
+};
+
+// Site s's populations into the sums of rho (deviations: less rho0) and of the momentum, over pairs of opposite
+// velocities: c_i (n_i - n_-i), whose products with c in {1, 2, 4} are exact.
 template <int LAT, int S>
-__device__ __forceinline__ void site_sums(const DevSim& p, int src, long long s, double (&acc)[4])
+__device__ __forceinline__ void site_sums(const DevSim& p, int src, long long s, Sum3& rho, Sum3 (&j)[3])
 {
     using L = Lat<LAT>;
     using C = Codec<S>;
@@ -3364,44 +3384,52 @@ __device__ __forceinline__ void site_sums(const DevSim& p, int src, long long s,
 #pragma unroll
     for (int i = 1; i < L::Q; ++i) v[i] = pop_raw<LAT, S, float>(p, src, i, s);
     const float2 r0 = cp<float2>(p.pop0[src])[s];
-    float hi = r0.x, lo = r0.y;
+    rho.add(r0.x);
+    rho.add(r0.y);
     if (C::LOC) {  // the decoded values fl(stored + sender's reference), see pop_full
         const int x = int(s % p.nx), y = int((s / p.nx) % p.ny), z = int(s / ((long long)p.nx * p.ny));
 #pragma unroll
         for (int i = 1; i < L::Q; ++i)
             v[i] = __fadd_rn(v[i], p.wref[src][L::shell(i) * p.N + sender<LAT>(p, x, y, z, i)]);
-        acc2(hi, lo, p.wref[src][s]);
+        rho.add(p.wref[src][s]);
     }
-    float jh[3] = {0.f, 0.f, 0.f}, jl[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int i = 1; i < L::Q; i += 2) {
-        acc2(hi, lo, v[i]);
-        acc2(hi, lo, v[i + 1]);
+        rho.add(v[i]);
+        rho.add(v[i + 1]);
         float d, e;
         two_sum(v[i], -v[i + 1], d, e);
         const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
 #pragma unroll
         for (int a = 0; a < L::D; ++a)
             if (c[a]) {
-                acc2(jh[a], jl[a], float(c[a]) * d);  // exact: c is 1, 2 or 4
-                jl[a] = __fadd_rn(jl[a], float(c[a]) * e);
+                j[a].add(float(c[a]) * d);
+                j[a].low(float(c[a]) * e);
             }
     }
-    acc[0] += (double(hi) + double(lo)) + (C::DEV && !C::LOC ? p.rho0 : 0.0);
-#pragma unroll
-    for (int a = 0; a < L::D; ++a) acc[1 + a] += double(jh[a]) + double(jl[a]);
 }
 
 template <int LAT, int S>
 __global__ void __launch_bounds__(kRedBlock, 2) k_red_partial(DevSim p, int src, double* part)
 {
     using L = Lat<LAT>;
+    using C = Codec<S>;
     __shared__ double sm[4][RED_BLOCK];
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (long long s = blockIdx.x * (long long)RED_BLOCK + threadIdx.x; s < p.N; s += (long long)RED_GRID * RED_BLOCK) {
-        if constexpr (Codec<S>::EXACT) {
-            site_sums<LAT, S>(p, src, s, acc);
-        } else {
+    const long long s0 = blockIdx.x * (long long)RED_BLOCK + threadIdx.x, ds = (long long)RED_GRID * RED_BLOCK;
+    bool wide = !C::EXACT;  // FP64 storage, or sums that leave the range of floats
+    if constexpr (C::EXACT) {
+        Sum3 rho = {0.f, 0.f, 0.f}, j[3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+        for (long long s = s0; s < p.N; s += ds) site_sums<LAT, S>(p, src, s, rho, j);
+        const long long sites = s0 < p.N ? (p.N - s0 + ds - 1) / ds : 0;
+        wide = !(rho.finite() && j[0].finite() && j[1].finite() && j[2].finite());
+        acc[0] = rho.value() + (C::DEV && !C::LOC ? double(sites) * p.rho0 : 0.0);
+#pragma unroll
+        for (int a = 0; a < L::D; ++a) acc[1 + a] = j[a].value();
+    }
+    if (wide) {
+        for (double& a : acc) a = 0.0;
+        for (long long s = s0; s < p.N; s += ds) {
 #pragma unroll
             for (int i = 0; i < L::Q; ++i) {
                 const double v = pop_full<LAT, S>(p, src, i, s);
