@@ -21,6 +21,7 @@
 #include "lbm_batch.h"
 #include "lbm_common.h"
 #include "lbm_lattice.h"
+#include "lbm_plan.h"
 
 using namespace lbm;
 
@@ -217,17 +218,6 @@ size_t bytes_per_site(int lattice, int storage, size_t* ssize_out = nullptr)
     return 2 * Q * ssize + rest + wref + tsize * (1 + 3 + 3 + naux) + usize * (4 * 3 + 2 * 3 + 2 * 3);
 }
 
-// whether x-neighbouring sites (2k, 2k + 1) are aligned words of every field plane
-bool pairs_of_sites(const int64_t dims[3]) { return dims[0] % 2 == 0; }
-// Whether the pairwise collision takes tiles of 64 x 4 sites (else 32 x 8): where they pad nx by at most a
-// fifth more.  Measured, 64 / 32 wide: 256^3 1.17 / 1.59 ms, 192^3 0.50 / 0.56, 160^3 (padded by a fifth)
-// 0.333 / 0.329, 128^3 0.155 / 0.160, 96^3 (a third) 0.087 / 0.076, 48^3 14 / 15 us.
-bool wide_tiles(const int64_t dims[3])
-{
-    const int64_t w32 = (dims[0] + 31) / 32 * 32, w64 = (dims[0] + 63) / 64 * 64;
-    return 5 * w64 <= 6 * w32;
-}
-
 int validate(int lattice, const int64_t dims[3], int storage)
 {
     if (lattice != LBM_D2Q21 && lattice != LBM_D3Q59) return LBM_E_INVALID_ARG;
@@ -240,9 +230,9 @@ int validate(int lattice, const int64_t dims[3], int storage)
     const double N = double(dims[0]) * double(dims[1]) * double(dims[2]);
     const int Q = lattice == LBM_D3Q59 ? 59 : 21;
     if (N * Q > 9.0e18 / 8.0) return LBM_E_INVALID_ARG;
-    // site indices inside a plane stack are 32-bit in the streaming kernel; the tiled
-    // kernels' grid has ceil(ny / 16) <= 65535 rows
-    if (N >= 2147483648.0 || dims[1] > 65535 * 8) return LBM_E_INVALID_ARG;
+    // site indices inside a plane stack are 32-bit in the streaming kernel; the tiled kernels' grids have
+    // ceil(ny / 8) rows of CTAs (wide_tiles keeps to lattices whose four-row tiles fit)
+    if (N >= 2147483648.0 || dims[1] > kGridRows * 8) return LBM_E_INVALID_ARG;
     return LBM_OK;
 }
 

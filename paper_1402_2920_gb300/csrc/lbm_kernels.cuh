@@ -28,6 +28,7 @@
 
 #include "lbm_common.h"
 #include "lbm_lattice.h"
+#include "lbm_plan.h"
 
 namespace lbm {
 
@@ -2500,7 +2501,7 @@ __device__ __forceinline__ void acc2_2(float2& hi, float2& lo, float2 v)
 // stencil and one in flight, and two stages of the tile's own inputs.
 template <int W>
 struct PairCollidePlan {
-    static constexpr int TX = W, TY = 256 / W, NT = TX * TY / 2, SITES = TX * TY;
+    static constexpr int TX = W, TY = pair_tile_rows(W), NT = TX * TY / 2, SITES = TX * TY;
     static constexpr int RX = TX + 4, RY = TY + 4, RP = RX * RY, NP = 3;
     static constexpr int R = 6;
     static constexpr int NOWN = 27;  // Sigma's local part (6), Xi' (10), u, j0', f, rho - rho0, rho_lo
