@@ -1200,7 +1200,7 @@ __device__ __forceinline__ void b_sweep(const DevSim& p, int pair, const Blk bid
     U* unew = mp<U>(p.uit[pair][cur ^ 1]);
     const U c1 = U(p.us[pair].c1), c2 = U(p.us[pair].c2);  // this sweep's update (see k_us_ctl)
     U* dvec = mp<U>(p.dvec[pair]);
-    const bool use_d = c1 != U(0), keep_d = p.cheb != 0;
+    const bool use_d = c1 != U(0), keep_d = p.cheb != 0 && keeps_update(p.us[pair]);
     // the thread's own site (stage J)
     const int ix = tid % TX, iy = tid / TX;
     const int gx = x0 + ix, gy = y0 + iy;
@@ -1618,7 +1618,7 @@ __device__ __forceinline__ void b_sweep_pm(const DevSim& p, int pair, const Blk 
     float* unew = mp<float>(p.uit[pair][cur ^ 1]);
     const float c1 = float(p.us[pair].c1), c2 = float(p.us[pair].c2);  // this sweep's update (see k_us_ctl)
     float* dvec = mp<float>(p.dvec[pair]);
-    const bool use_d = c1 != 0.f, keep_d = p.cheb != 0, use_j = p.rtol != 0.0;
+    const bool use_d = c1 != 0.f, keep_d = p.cheb != 0 && keeps_update(p.us[pair]), use_j = p.rtol != 0.0;
     // the thread's own site (stage J)
     const int ix = tid % TX, iy = tid / TX;
     const int gx = x0 + ix, gy = y0 + iy;

@@ -79,6 +79,10 @@ LBM_HD void cheb_first(UsolveState& u)
     u.c2 = 1.0 / (1.0 - u.cheb_delta);
 }
 
+// Whether the sweep leaves its update for the next one: only a Chebyshev sweep is followed by one that reads it
+// (c1 != 0).  The vector is 12 of a plain FP32 sweep's 60 bytes per site.
+LBM_HD bool keeps_update(const UsolveState& u) { return u.mode == 1; }
+
 // A solve's start: spectrum bound g, and its first update.  `run` is the run's last solve, which a scratch
 // solve reads too: what it does depends on the run's state alone.  cheb, omega, maxit: see DevSim.
 LBM_HD void usolve_open(UsolveState& u, const UsolveState& run, int cheb, double omega, int maxit, double g)

@@ -40,11 +40,16 @@ int main(int, char** a)
         for (int k = 0; k < M; ++k) r[k] *= first / total;
         usolve_open(u, u, cheb, 0.0, maxit, g);
         const int opened = (u.opened & US_PLAIN) != 0;
+        int missing = 0, unread = 0;  // sweeps that read an update none left; plain sweeps that leave theirs
+        bool kept = false;
         while (u.iter < 1000) {
             double norm = 0.0;
             for (int k = 0; k < M; ++k) norm += std::fabs(r[k]);
             seed = seed * 1664525u + 1013904223u;
             norm += rounding * (seed >> 8) / 16777216.0;  // what the rounding of u puts into the residual
+            missing += u.c1 != 0.0 && !kept;
+            kept = keeps_update(u);
+            unread += kept && u.mode != 1;
             for (int k = 0; k < M; ++k) {
                 d[k] = u.c1 * d[k] + u.c2 * r[k];
                 r[k] -= (1.0 - J[k]) * d[k];
@@ -57,7 +62,7 @@ int main(int, char** a)
             if (stop) break;
         }
         u.iters_last = u.iter;
-        std::printf("%d %d\n", opened, u.iter);
+        std::printf("%d %d %d %d\n", opened, u.iter, missing, unread);
     }
     return 0;
 }
@@ -80,6 +85,7 @@ def model(tmp_path_factory):
         out = subprocess.run([str(exe)] + [str(v) for v in (cheb, maxit, g, smooth, rough, first, decline, solves, rounding)],
                              check=True, capture_output=True, text=True).stdout
         rows = [[int(v) for v in line.split()] for line in out.splitlines()]
+        assert not any(r[2] or r[3] for r in rows)  # the update vector: written before it is read, by no plain sweep
         return [r[1] for r in rows], [r[0] for r in rows]
 
     return run
