@@ -710,18 +710,20 @@ int lbm_create(int lattice, const int64_t dims[3], const lbm_eos* eos, const lbm
     s->eos = *eos;
     s->prm = *params;
 
-    const bool us64 = usolve_f64(*params);
+    const bool f64 = params->storage == LBM_STORE_F64;
+    const bool us64 = f64 || params->usolve_precision == LBM_USOLVE_F64;
     const bool read_pops = params->gamma != 0.0;
     bool ok = lattice == LBM_D3Q59 ? get_kernels_d3q59(params->storage, us64, read_pops, &s->kt)
                                    : get_kernels_d2q21(params->storage, us64, read_pops, &s->kt);
     if (!ok) { delete s; return LBM_E_INVALID_ARG; }
-    if (const int pc = pair_class(lattice, dims, *params)) {  // the kernels on pairs of sites
+    // the kernels on pairs of sites need pairs that stay aligned words: nx even
+    if (s->kt.pair_derivs && pairs_of_sites(dims)) {
         KernelTable& kt = s->kt;
         kt.derivs = kt.pair_derivs;
         kt.kb_derivs = kt.kb_pair_derivs;
         kt.tile[TK_DERIVS] = kt.tile_pair_derivs;
         kt.smem_derivs = kt.smem_pair_derivs;
-        const PairCollide& c = kt.pair_collide[pc - 1];
+        const PairCollide& c = kt.pair_collide[wide_tiles(dims) ? 1 : 0];
         kt.collide = c.collide;
         kt.kb_collide = c.kb_collide;
         kt.tile[TK_COLLIDE] = c.tile;
@@ -1284,6 +1286,20 @@ struct Batch {
     cudaGraph_t g = nullptr;
     cudaGraphExec_t x = nullptr;
 };
+
+int batch_key(int lattice, const int64_t dims[3], const lbm_params& prm)
+{
+    const bool us64 = prm.storage == LBM_STORE_F64 || prm.usolve_precision == LBM_USOLVE_F64;
+    const int combo = (((lattice * 16 + prm.storage) * 2 + (us64 ? 1 : 0)) * 2 + (prm.gamma != 0.0 ? 1 : 0)) * 3 +
+                      (pairs_of_sites(dims) ? (wide_tiles(dims) ? 2 : 1) : 0);
+    int64_t n = dims[0] * dims[1] * (lattice == LBM_D3Q59 ? dims[2] : 1);
+    int size_class = 0;
+    while (n >= 4) {
+        n >>= 2;
+        ++size_class;
+    }
+    return combo * 64 + size_class;
+}
 
 int batch_key_of(const lbm_sim* s) { return batch_key(s->lattice, s->dims, s->prm); }
 

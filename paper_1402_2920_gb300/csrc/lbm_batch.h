@@ -12,12 +12,15 @@
 
 #include "lbm.h"
 #include "lbm_common.h"
-#include "lbm_plan.h"
 
 namespace lbm {
 
 struct Batch;
 
+// Batch key of a simulation: its kernel combination and its size class (sites within a factor
+// of 4).  Simulations batch together only when their keys are equal: a batch steps in lockstep,
+// so a small simulation beside a much larger one would wait for it at every stage.
+int batch_key(int lattice, const int64_t dims[3], const lbm_params& prm);
 int batch_key_of(const lbm_sim* s);
 
 // A batch for the key of `proto` whose launches go to `stream`.
