@@ -1287,6 +1287,10 @@ struct Batch {
     cudaGraphExec_t x = nullptr;
 };
 
+// The class of nx (odd, or the pairwise collision's tile width) tells batches apart for every combination, also where
+// no kernel depends on it: a batch steps in lockstep, and up to three smaller ones on their own streams overlap.
+// Measured, ms against one batch: 15 requests of 96^2, 113^2, 120^2 54.5 / 64.5, of 352^2, 480^2, 511^2 200 / 212;
+// 12 of 40^3, 48^3, 51^3 with 16-bit populations 69.9 / 72.7, with FP32 n_i 132 / 134.
 int batch_key(int lattice, const int64_t dims[3], const lbm_params& prm)
 {
     const bool us64 = prm.storage == LBM_STORE_F64 || prm.usolve_precision == LBM_USOLVE_F64;

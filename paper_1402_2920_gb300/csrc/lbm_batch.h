@@ -17,7 +17,7 @@ namespace lbm {
 
 struct Batch;
 
-// Batch key of a simulation: its kernel combination and its size class (sites within a factor
+// Batch key of a simulation: its kernel combination, its class of nx and its size class (sites within a factor
 // of 4).  Simulations batch together only when their keys are equal: a batch steps in lockstep,
 // so a small simulation beside a much larger one would wait for it at every stage.
 int batch_key(int lattice, const int64_t dims[3], const lbm_params& prm);
