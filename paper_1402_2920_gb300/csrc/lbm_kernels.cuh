@@ -3303,6 +3303,7 @@ template <int LAT, typename T, typename U>
 __global__ void k_fields_out(DevSim p, int pair, double* rho_out, double* u_out)
 {
     using L = Lat<LAT>;
+    if (p.us[pair].running) return;  // launched ahead, and the solve goes on
     const long long s = gtid();
     if (s >= p.N) return;
     const T rs = phys<T>(p).rho0 + cp<T>(p.rho)[s];
