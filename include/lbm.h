@@ -193,7 +193,8 @@ int lbm_stats_get(lbm_sim* sim, lbm_stats* out);
  * times back to back, after one untimed launch, between two CUDA events on the
  * simulation's stream; ms_out[k] receives the average milliseconds per launch of
  * kernel k for k < n, in the order 0 moments (S1), 1 force (S2), 2 one u-solve
- * sweep (S3-S6), 3 derivatives (S8-S11, site-local parts), 4 collision and
+ * sweep (S3-S6; with usolve_chebyshev a Chebyshev sweep after the first, which
+ * moves more than a plain one), 3 derivatives (S8-S11, site-local parts), 4 collision and
  * streaming (S11-S12).  Only per-step temporaries are written,
  * so the simulation's state is unchanged.  Synchronises. */
 int lbm_profile(lbm_sim* sim, int reps, double* ms_out, int n);

@@ -1129,6 +1129,18 @@ int lbm_profile(lbm_sim* s, int reps, double* ms_out, int n)
     LBM_CK(launch_tiled(s, TK_FORCE, dv, pair));
     LBM_CK(launch(s, s->kt.us_begin, 1, 32, dv, pair));
     const int alone = SWEEP_ALONE;
+    if (dv.cheb) {
+        // the sweep as a Chebyshev solve runs it after its first, which reads and writes the update vector (us_begin
+        // alone would leave c1 = 0: 60 instead of 72 bytes per site in FP32)
+        UsolveState u{};
+        LBM_CK(cudaMemcpyAsync(&u, &dv.us[pair], sizeof(u), cudaMemcpyDeviceToHost, s->stream));
+        LBM_CK(cudaStreamSynchronize(s->stream));
+        cheb_first(u);
+        usolve_next(u, 2, 0.0, 0.0);
+        LBM_CK(cudaMemcpyAsync(&dv.us[pair], &u, sizeof(u), cudaMemcpyHostToDevice, s->stream));
+        LBM_CK(cudaStreamSynchronize(s->stream));  // u lives on this stack
+        LBM_CK(cudaMemsetAsync(dv.dvec[pair], 0, 3 * size_t(dv.N) * s->kt.usize, s->stream));
+    }
     int rc = LBM_OK;
     for (int k = 0; k < 5 && rc == LBM_OK; ++k) {
         for (int r = 0; r <= reps && rc == LBM_OK; ++r) {
@@ -1152,6 +1164,11 @@ int lbm_profile(lbm_sim* s, int reps, double* ms_out, int n)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     (void)cudaGetLastError();
+    if (rc == LBM_OK && trace_mode()) {
+        UsolveState u{};
+        if (cudaMemcpy(&u, &dv.us[pair], sizeof(u), cudaMemcpyDeviceToHost) != cudaSuccess) rc = LBM_E_CUDA;
+        std::fprintf(stderr, "lbm profile sweep c1 %.4f c2 %.4f\n", u.c1, u.c2);
+    }
     // the scratch residual accumulators were left mid-loop: clear them; restore the warm start
     UsolveState u1{};
     if (rc == LBM_OK && cudaMemcpyAsync(&dv.us[1], &u1, sizeof(u1), cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
