@@ -1169,7 +1169,9 @@ int lbm_profile(lbm_sim* s, int reps, double* ms_out, int n)
         if (cudaMemcpy(&u, &dv.us[pair], sizeof(u), cudaMemcpyDeviceToHost) != cudaSuccess) rc = LBM_E_CUDA;
         std::fprintf(stderr, "lbm profile sweep c1 %.4f c2 %.4f\n", u.c1, u.c2);
     }
-    // the scratch residual accumulators were left mid-loop: clear them; restore the warm start
+    // the scratch solve's density ranges hold this state's (lbm_fields would widen its own with them): empty them; its
+    // residual accumulators were left mid-loop: clear them; restore the warm start
+    if (rc == LBM_OK && launch(s, s->kt.us_begin, 1, 32, dv, pair) != cudaSuccess) rc = LBM_E_CUDA;
     UsolveState u1{};
     if (rc == LBM_OK && cudaMemcpyAsync(&dv.us[1], &u1, sizeof(u1), cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
         rc = LBM_E_CUDA;
