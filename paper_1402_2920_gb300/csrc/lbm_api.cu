@@ -431,8 +431,9 @@ bool encode_plane_map(CUtensorMap* m, void* base, int ncomp, size_t esize, const
 
 // The sweep kernel: the tensor-copy (TMA) form, whose tensor maps need a 3D lattice with rows a
 // multiple of 16 bytes, or per-thread plane copies (2D, other sizes, or LBM_SWEEP_COPY=cp_async in
-// the environment).  The TMA form is the default: at three CTAs per SM it is the faster of the two
-// (0.395 against 0.402 ms at 256^3), the copies no longer issued by every thread.
+// the environment).  The two are close: Chebyshev sweep with tensor / per-thread copies, us, 256^3 368 / 366, 192^3 173 / 170,
+// 160^3 110 / 107, 128^3 61.6 / 59.5, 288 x 192 x 224 280 / 281.  The tensor form is the default: it wins on the
+// largest of these, and leaves the threads no copies to issue.
 void setup_sweep_maps(lbm_sim* s)
 {
     DevSim& dv = s->dev;

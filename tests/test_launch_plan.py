@@ -52,3 +52,12 @@ def test_grids_of_the_tallest_lattices_fit(tmp_path):
     # ... and the width is that of nx alone up to the last ny whose rows fit
     wide = {d[0]: int(line.split()[0]) for d, line in zip(dims, out) if d[1] == 262140}
     assert wide[34] == wide[64] == wide[128] == wide[256] == 64 and wide[4] == wide[66] == 32
+
+
+def test_tile_widths_of_the_pairwise_collision(tmp_path):
+    """64 wide where that pads nx by at most a fifth more than 32 wide."""
+    wide = (34, 62, 64, 98, 100, 128, 130, 160, 192, 256, 288)
+    narrow = (4, 32, 66, 90, 96)
+    out = _run(tmp_path, PROGRAM, "\n".join("%d 8 8" % nx for nx in wide + narrow))
+    got = {nx: int(line.split()[0]) for nx, line in zip(wide + narrow, out)}
+    assert all(got[nx] == 64 for nx in wide) and all(got[nx] == 32 for nx in narrow)
