@@ -604,16 +604,18 @@ static __device__ bool b_us_ctl(const DevSim& p, int pair)
     u.sweeps_total += 1;
     u.cur ^= 1;
     const bool bad = !isfinite(r);
-    const bool conv = !bad && r <= p.tol + p.rtol * jm;
+    const double lim = p.tol + p.rtol * jm;
+    const bool conv = !bad && r <= lim;
     const bool stop = conv || bad || u.iter >= p.maxit;
     if (bad) atomicOr(p.status, STB_USOLVE_NAN);
     else if (stop && !conv) atomicOr(p.status, STB_USOLVE_CAP);
     u.resid_bits = 0ull;
     u.jmax_bits = 0ull;
-    if (p.cheb && !bad) usolve_next(u, p.cheb, r, p.tol + p.rtol * jm);
+    if (p.cheb && !stop) usolve_next(u, p.cheb, r, lim);
     u.resid_last = r;
     u.resid_min = r < u.resid_min ? r : u.resid_min;
     if (stop) {
+        usolve_end(u);
         u.iters_last = u.iter;
         u.iters_max = u.iter > u.iters_max ? u.iter : u.iters_max;
         u.converged = conv ? 1 : 0;

@@ -59,7 +59,7 @@ struct UsolveState {
 // staying plain while the residual halves / these rules: 256^3 spinodal steps 6-25 5.95 / 6.35 / 5.95, steps 41-48
 // 2.4 / 2.0 / 2.0; mean of 512^2 spinodals in a flow over 60 steps - / 4.90 / 4.34; 128^3 droplets in a flow over
 // 200 steps 6 / 2.53 / 2.53.
-enum OpenedBits { US_PLAIN = 1, US_SMOOTH = 2, US_CALM = 1 << 4, US_COUNT = 1 << 8, US_CHEB = 1 << 16 };
+enum OpenedBits { US_PLAIN = 1, US_SMOOTH = 2 };  // bits 4-7 calm, 8-15 count, 16-23 dear (usolve_open)
 constexpr int kPlainOpenMost = 5, kCalm = 6, kWait = 4, kRecheck = 16;
 constexpr double kPlainNear = 4.0, kStallNear = 2.0;
 
@@ -99,7 +99,7 @@ LBM_HD void usolve_open(UsolveState& u, const UsolveState& run, int cheb, double
     u.tma = 0;
     u.resid_min = 1e300;
     u.resid_last = 1e300;
-    int calm = last / US_CALM % 16, count = last / US_COUNT % 256, dear = last / US_CHEB % 256;
+    int calm = last >> 4 & 15, count = last >> 8 & 255, dear = last >> 16 & 255;
     calm = n == 0 ? 0 : n <= kPlainOpenMost ? calm + 3 : n == kPlainOpenMost + 1 ? calm + 1 : 0;
     calm = calm < kCalm ? calm : kCalm;
     bool smooth = last & US_SMOOTH, plain;
@@ -116,7 +116,7 @@ LBM_HD void usolve_open(UsolveState& u, const UsolveState& run, int cheb, double
         count = kWait;
     }
     plain = plain && cheb == 1 && n > 0 && maxit > 2 * kPlainOpenMost;
-    u.opened = (plain ? US_PLAIN : 0) + (smooth ? US_SMOOTH : 0) + calm * US_CALM + count * US_COUNT + dear * US_CHEB;
+    u.opened = (plain ? US_PLAIN : 0) | (smooth ? US_SMOOTH : 0) | calm << 4 | count << 8 | dear << 16;
     if (plain) {
         u.mode = 2;
         plain_sweep(u);
@@ -129,29 +129,38 @@ LBM_HD void usolve_open(UsolveState& u, const UsolveState& run, int cheb, double
     }
 }
 
-// The next update of an accelerated solve after sweep u.iter, of residual r (finite) and tolerance lim: Chebyshev
-// semi-iteration for the real spectrum [1 - g, 1] of I - A, or plain.  resid_last holds the residual of
+// An accelerated solve's end after sweep u.iter: one that a plain opening brought there in two sweeps was smooth.
+LBM_HD void usolve_end(UsolveState& u)
+{
+    if (u.iter == 2 && (u.opened & US_PLAIN)) u.opened |= US_SMOOTH;
+}
+
+// The next update of an accelerated solve that goes on after sweep u.iter, of residual r (finite) and tolerance lim:
+// Chebyshev semi-iteration for the real spectrum [1 - g, 1] of I - A, or plain.  resid_last holds the residual of
 // the sweep before.  A residual four times above the best one so far means the spectral bound was too small: plain
-// sweeps from there on (mode 0).
+// sweeps from there on (mode 0).  (One thread, which waits for the few FP64 units at each operation: what decides
+// comes in products, q = r / r0, and the cheapest first.)
 LBM_HD void usolve_next(UsolveState& u, int cheb, double r, double lim)
 {
-    const double q = r / u.resid_last;
     if (u.mode == 1 && r > 4.0 * u.resid_min) u.mode = 0;
     bool plain = u.mode == 0;
     if (cheb == 1) {
-        const bool opening = (u.opened & US_PLAIN) && (u.mode == 2 || u.iter <= 2);
-        if (opening && u.iter == 1) {
+        const double r0 = u.resid_last;
+        if (!(u.opened & US_PLAIN) || (u.mode != 2 && u.iter > 2)) {
+            // stalled: no progress of the size that Chebyshev makes (its factor is below 1 / sigma)
+            plain = plain || u.mode == 2 || (r <= kStallNear * lim && r > 0.5 * r0 && r * u.cheb_sigma > r0);
+        } else if (u.iter == 1) {
             plain = (u.opened & US_SMOOTH) || r <= kPlainNear * lim;
-        } else if (opening) {
+        } else {
             // near: at the rounding of u, where q tells nothing (g bounds the plain sweeps left there), or halving;
             // smooth: q against Chebyshev's factor sigma - sqrt(sigma^2 - 1), to its second order in 1 / sigma
-            const bool near = r <= kPlainNear * lim && (q <= 0.5 || u.gain <= 0.8);
-            const bool smooth = q * (2.0 * u.cheb_sigma - 0.5 / u.cheb_sigma) <= 1.0 || near;
-            if (u.iter == 2) u.opened = (u.opened & ~US_SMOOTH) | (smooth ? US_SMOOTH : 0);
-            plain = plain || near || q * q * r <= lim;
-        } else {
-            // stalled: no progress of the size that Chebyshev makes (its factor is below 1 / sigma)
-            plain = plain || u.mode == 2 || (r <= kStallNear * lim && q > 0.5 && q * u.cheb_sigma > 1.0);
+            const double sg = u.cheb_sigma;
+            const bool near = r <= kPlainNear * lim && (u.gain <= 0.8 || r <= 0.5 * r0);
+            if (u.iter == 2) {
+                const bool smooth = near || r * (4.0 * sg * sg - 1.0) <= 2.0 * sg * r0;
+                u.opened = (u.opened & ~US_SMOOTH) | (smooth ? US_SMOOTH : 0);
+            }
+            plain = plain || near || r * r * r <= lim * r0 * r0;  // q^2 r: the residual two sweeps on
         }
     }
     if (plain) {

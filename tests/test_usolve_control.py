@@ -56,7 +56,8 @@ int main(int, char** a)
             }
             u.iter += 1;
             const bool stop = norm <= lim;
-            if (cheb) usolve_next(u, cheb, norm, lim);
+            if (cheb && !stop) usolve_next(u, cheb, norm, lim);
+            if (stop) usolve_end(u);
             u.resid_last = norm;
             u.resid_min = norm < u.resid_min ? norm : u.resid_min;
             if (stop) break;
