@@ -117,7 +117,8 @@ def _kernel_sources_sha():
     h = hashlib.sha256()
     cdir = os.path.join(ROOT, "paper_1402_2920_gb300", "csrc")
     for name in sorted(os.listdir(cdir)):  # the files that define the kernels
-        if not (name.startswith("kernels_") or name in ("lbm_kernels.cuh", "lbm_lattice.h", "lbm_common.h")):
+        if not (name.startswith("kernels_") or name in ("lbm_kernels.cuh", "lbm_lattice.h", "lbm_common.h",
+                                                          "lbm_plan.h", "lbm_usolve.h")):
             continue
         with open(os.path.join(cdir, name), "rb") as fh:
             h.update(name.encode())

@@ -575,8 +575,8 @@ void choose_zb(lbm_sim* s)
 
 // S1-S8 on the current populations with the scratch j~ pair, and the fields to device memory.  The sweeps are
 // launched kAhead at a time, the fields' kernel behind them: sweeps that come after the solve has stopped
-// return at once, and one copy tells whether it has.  (One sweep and one copy in turn left the device idle
-// for the host's round trip at each sweep.)
+// return at once, a fields' kernel before it has too, and one copy tells whether it has.  (One sweep and one copy in turn
+// left the device idle for the host's round trip at each sweep.)
 int run_fields(lbm_sim* s, double* rho, double* u, HostView* v)
 {
     constexpr int kAhead = 4;

@@ -1594,10 +1594,12 @@ struct SweepPmPlan {
 //     barrier per phase instead of two, at three CTAs per SM as before (75 KB each).
 //   - Two tensor copies per plane (all components of a field in one box) instead of four, and the
 //     z-derivative sums roll through their own updates instead of being copied from plane to plane.
-// Measured: 395 -> 317 us at 256^3, 119 -> 93 at 160^3, 66 -> 64 at 128^3 (one wave); the force kernel 231 -> 250 us at 256^3,
-// once per step.  72 bytes per site, 0.57 of the measured copy bandwidth at 256^3; bound by shared memory
-// (4.0 wavefronts per site) and the latency between its barriers.  Tried on the way: two sites per thread on 32 x 16 tiles
-// (16 warps per SM) 366 us, 512 threads on 32 x 16 tiles 397 us, packed stage Q alone 387 us.
+// Measured, b_sweep / this kernel: a Chebyshev sweep that reads and writes the update vector (64 / 72 bytes per site)
+// 403 / 365 us at 256^3, 137 / 109 at 160^3, 77 / 62 at 128^3 (one wave), 0.40 / 0.49 of the measured copy bandwidth at
+// 256^3; a plain sweep (40 / 48) 380 / 305, 131 / 95, 72 / 53.  The force kernel 231 / 250 us at 256^3, once per step.
+// Bound by shared memory (4.0 wavefronts per site) and the latency between its barriers.  Tried on the way, against
+// 317 us for a first Chebyshev sweep, which writes the vector alone: two sites per thread on 32 x 16 tiles (16 warps per SM)
+// 366 us, 512 threads on 32 x 16 tiles 397 us, packed stage Q alone 387 us.
 template <bool TMA>
 __device__ __forceinline__ void b_sweep_pm(const DevSim& p, int pair, const Blk bid)
 {
